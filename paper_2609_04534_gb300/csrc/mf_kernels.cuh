@@ -889,120 +889,186 @@ __global__ void __launch_bounds__(N * N * CB, MINB) apply_general_batch(ApplyBat
 // ---------------------------------------------------------------------------------------
 // Duplicate summation y <- G G^T y (Sec. 4: embedding G and assembly G^T) in the canonical
 // order of the dimension-split sweeps of Sec. 3: the copies of a node are summed pairwise
-// along x, then the x-sums along y, then along z.  One thread per global node; each copy
-// is read and written by exactly one thread, so no atomics and no races.
-// ---------------------------------------------------------------------------------------
-__device__ __forceinline__ int copies_1d(long long I, int ncell, int k, int* cell, int* loc) {
-  const long long c = I / k;
-  if (I - c * k == 0) {
-    if (c == 0) { cell[0] = 0; loc[0] = 0; return 1; }
-    if (c == ncell) { cell[0] = ncell - 1; loc[0] = k; return 1; }
-    cell[0] = (int)c - 1; loc[0] = k;
-    cell[1] = (int)c; loc[1] = 0;
-    return 2;
-  }
-  cell[0] = (int)c; loc[0] = (int)(I - c * k);
-  return 1;
-}
-
+// along x, then the x-sums along y, then along z.  Each node belongs to its lowest copy (the
+// cell with the smaller index in every direction), and that copy's lane reads and writes all
+// of its copies, so no atomics and no races.
+//
+// A warp takes rows (local node (i, j, k)) of a tile, lane = cell: its own copies are one
+// contiguous 32-element row, and the copies across a face are the row of the opposite local
+// node, shifted by one cell inside the tile (3 of 4 lanes along x and y, half along z) and in
+// the next tile for the rest.  In a tile away from the low mesh faces only the rows with
+// i, j, k >= 1 and at least one of them K own shared nodes, every lane of them is at work, and
+// a row's kind (which faces it lies on) is uniform in the warp.  The tiles on a low mesh face
+// get further warps for the rows with a zero index, for the lanes on that face.
+// Bound by the copies' traffic (each read and written once).  Measured on one GB300 against a
+// kernel with one thread per node along a row of nodes, which this one replaced (it spent 77
+// instructions per DoF on finding the copies, and half-used sectors in FP32): FP64 Q1 184^3
+// 0.157 -> 0.131 ms, Q4 74^3 0.232 -> 0.125 ms (5.1 TB/s), Q8 41^3 0.234 -> 0.115 ms;
+// FP32 Q4 64^3 0.153 -> 0.050 ms; Q2 8^3 4.4 -> 4.3 us.
 // avg = 1: the average of the copies instead of their sum (mf_make_consistent): the sum in
 // the same canonical order times 1/multiplicity (a power of two, so exact), and no Dirichlet
 // mask.
-template <typename T, int N>
-__global__ void dss_kernel(T* __restrict__ y, GridInfo g, int avg) {
-  constexpr int K = N - 1, N2 = N * N, N3 = N2 * N;
-  const long long NX = (long long)g.nx * K + 1, NY = (long long)g.ny * K + 1, NZ = (long long)g.nz * K + 1;
-  const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (gid >= NX * NY * NZ) return;
-  const long long I = gid % NX, J = (gid / NX) % NY, L = gid / (NX * NY);
-  int cx[2], ix[2], cy[2], iy[2], cz[2], iz[2];
-  const int mx = copies_1d(I, g.nx, K, cx, ix);
-  const int my = copies_1d(J, g.ny, K, cy, iy);
-  const int mz = copies_1d(L, g.nz, K, cz, iz);
-  const bool bnd = !avg && g.bc && (I == 0 || I == NX - 1 || J == 0 || J == NY - 1 || L == 0 || L == NZ - 1);
-  if (mx * my * mz == 1 && !bnd) return;
-  long long addr[8];
-  T s = T(0);
-  T sz[2];
-  for (int zz = 0; zz < mz; ++zz) {
-    T sy[2];
-    for (int yy = 0; yy < my; ++yy) {
-      T sx = T(0);
-      for (int xx = 0; xx < mx; ++xx) {
-        const long long ad = native_index(g, N3, cx[xx], cy[yy], cz[zz], ix[xx] + N * iy[yy] + N2 * iz[zz]);
-        addr[xx + 2 * (yy + 2 * zz)] = ad;
-        const T v = y[ad];
-        sx = (xx == 0) ? v : sx + v;
-      }
-      sy[yy] = sx;
-    }
-    sz[zz] = (my == 2) ? sy[0] + sy[1] : sy[0];
-  }
-  s = (mz == 2) ? sz[0] + sz[1] : sz[0];
-  if (avg) s = s * (T(1) / T(mx * my * mz));
-  if (bnd) s = T(0);
-  for (int zz = 0; zz < mz; ++zz)
-    for (int yy = 0; yy < my; ++yy)
-      for (int xx = 0; xx < mx; ++xx) y[addr[xx + 2 * (yy + 2 * zz)]] = s;
-}
+// ---------------------------------------------------------------------------------------
+constexpr int DSS_THREADS = 256;
+template <int N>
+struct DssCfg {
+  static constexpr int K = N - 1, E = K - 1;
+  // Rows of an inner tile by kind: (K-1)^2 on each of the three faces, K-1 on each edge, the
+  // vertex.  A warp takes one chunk of U rows along a line (U loads in flight per copy and
+  // lane), CL chunks per line, so that a copy's address is one pointer plus constant offsets.
+  // (A loop over chunks made the compiler keep every kind's pointers: 160 registers.)
+  static constexpr int U = E < 1 ? 1 : (E <= 4 ? E : (E + 1) / 2), CL = (E + U - 1) / U;
+  static constexpr int CHUNKS = 1 + 3 * CL + 3 * CL * E;
+  static constexpr int LOW = N * N * N - K * K * K; // rows with a zero index
+};
 
-// The same duplicate summation with the global nodes of (J, L) rows per block and the cells
-// fastest across threads: thread (i, cx) takes node I = cx k + i (for i = 0 the extra column
-// cx = nx takes the row's last node I = nx k), so for one i consecutive threads read
-// consecutive lanes of a tile (whole 32-byte sectors); J and L come from the grid and a
-// block loops over DSS_ROWS_Y-strided rows (no division per thread, few blocks).  Same sums
-// in the same canonical order as dss_kernel, so bitwise equal.
-constexpr int DSS_ROW_THREADS = 128, DSS_ROWS_Y = 32;
-template <typename T, int N>
-__global__ void __launch_bounds__(DSS_ROW_THREADS) dss_row_kernel(T* __restrict__ y, GridInfo g, int avg, int cxb) {
-  constexpr int K = N - 1, N2 = N * N, N3 = N2 * N;
-  const int i = blockIdx.x / cxb;                                       // local x index
-  const int cxs = (blockIdx.x - i * cxb) * DSS_ROW_THREADS + threadIdx.x; // cell column
-  if (cxs > g.nx || (i > 0 && cxs == g.nx)) return;
-  const int NYn = g.ny * K + 1, NZn = g.nz * K + 1;
-  int cx[2], ix[2];
-  int mx;
-  if (cxs == g.nx) { mx = 1; cx[0] = g.nx - 1; ix[0] = K; }            // I = nx k, the last node
-  else if (i == 0 && cxs > 0) { mx = 2; cx[0] = cxs - 1; ix[0] = K; cx[1] = cxs; ix[1] = 0; }
-  else { mx = 1; cx[0] = cxs; ix[0] = i; }
-  const bool bx = (i == 0 && cxs == 0) || cxs == g.nx; // on the x = 0 or x = 1 face
-  for (int L = blockIdx.z; L < NZn; L += gridDim.z) {
-    int cz[2], iz[2];
-    const int mz = copies_1d(L, g.nz, K, cz, iz);
-    for (int J = blockIdx.y; J < NYn; J += gridDim.y) {
-      int cy[2], iy[2];
-      const int my = copies_1d(J, g.ny, K, cy, iy);
-      const bool bnd = !avg && g.bc && (bx || J == 0 || J == NYn - 1 || L == 0 || L == NZn - 1);
-      if (mx * my * mz == 1 && !bnd) continue;
-      long long addr[8];
+// What a lane needs to find and sum the copies of its nodes.
+struct DssLane {
+  long long o[3]; // element distance to the copy across the high x / y / z face
+  bool h[3];      // whether there is one
+  bool mask;      // constrained nodes are zeroed
+  int avg;
+};
+
+// `count` (<= U) rows of one kind (A / B / C: on the high x / y / z face of the cell), ST
+// elements apart from y[0]; low: the rows lie on a low mesh face.
+template <typename T, bool A, bool B, bool C, int U, int ST>
+__device__ __forceinline__ void dss_rows(T* __restrict__ y, const DssLane& d, int count, bool low) {
+  const bool X = A && d.h[0], Y = B && d.h[1], Z = C && d.h[2];
+  const bool zero = d.mask && (low || (A && !X) || (B && !Y) || (C && !Z));
+  if (!(X || Y || Z || zero)) return;
+  T v[2][2][2][U];
+#pragma unroll
+  for (int c = 0; c <= (C ? 1 : 0); ++c)
+#pragma unroll
+    for (int b = 0; b <= (B ? 1 : 0); ++b)
+#pragma unroll
+      for (int a = 0; a <= (A ? 1 : 0); ++a) {
+        const T* p = y + (a ? d.o[0] : 0) + (b ? d.o[1] : 0) + (c ? d.o[2] : 0);
+        if (!zero && (a == 0 || X) && (b == 0 || Y) && (c == 0 || Z)) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (u < count) v[c][b][a][u] = p[u * ST];
+        }
+      }
+  T s[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    s[u] = T(0);
+    if (!zero) {
       T sz[2];
 #pragma unroll
-      for (int zz = 0; zz < 2; ++zz) {
-        if (zz >= mz) break;
+      for (int c = 0; c <= (C ? 1 : 0); ++c) {
         T sy[2];
 #pragma unroll
-        for (int yy = 0; yy < 2; ++yy) {
-          if (yy >= my) break;
-          T sx = T(0);
-#pragma unroll
-          for (int xx = 0; xx < 2; ++xx) {
-            if (xx >= mx) break;
-            const long long ad = native_index(g, N3, cx[xx], cy[yy], cz[zz], ix[xx] + N * iy[yy] + N2 * iz[zz]);
-            addr[xx + 2 * (yy + 2 * zz)] = ad;
-            const T v = y[ad];
-            sx = (xx == 0) ? v : sx + v;
-          }
-          sy[yy] = sx;
+        for (int b = 0; b <= (B ? 1 : 0); ++b) {
+          sy[b] = v[c][b][0][u];
+          if (A && X) sy[b] = v[c][b][0][u] + v[c][b][1][u];
         }
-        sz[zz] = (my == 2) ? sy[0] + sy[1] : sy[0];
+        sz[c] = sy[0];
+        if (B && Y) sz[c] = sy[0] + sy[1];
       }
-      T s = (mz == 2) ? sz[0] + sz[1] : sz[0];
-      if (avg) s = s * (T(1) / T(mx * my * mz));
-      if (bnd) s = T(0);
-      for (int zz = 0; zz < mz; ++zz)
-        for (int yy = 0; yy < my; ++yy)
-          for (int xx = 0; xx < mx; ++xx) y[addr[xx + 2 * (yy + 2 * zz)]] = s;
+      s[u] = sz[0];
+      if (C && Z) s[u] = sz[0] + sz[1];
+      if (d.avg) s[u] = s[u] * ((X ? T(0.5) : T(1)) * (Y ? T(0.5) : T(1)) * (Z ? T(0.5) : T(1)));
     }
+  }
+#pragma unroll
+  for (int c = 0; c <= (C ? 1 : 0); ++c)
+#pragma unroll
+    for (int b = 0; b <= (B ? 1 : 0); ++b)
+#pragma unroll
+      for (int a = 0; a <= (A ? 1 : 0); ++a) {
+        T* p = y + (a ? d.o[0] : 0) + (b ? d.o[1] : 0) + (c ? d.o[2] : 0);
+        if ((a == 0 || X) && (b == 0 || Y) && (c == 0 || Z)) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (u < count) p[u * ST] = s[u];
+        }
+      }
+}
+
+// Warp u of the launch: chunk u % CHUNKS of tile u / CHUNKS for u < nmain, then row by row the
+// LOW rows of the low-face tiles (the layer tz = 0, then ty = 0, then tx = 0 of the rest).
+template <typename T, int N>
+__global__ void __launch_bounds__(DSS_THREADS) dss_kernel(T* __restrict__ y, GridInfo g, int avg, long long nmain,
+                                                          long long nunits) {
+  using D = DssCfg<N>;
+  constexpr int K = N - 1, N2 = N * N, N3 = N2 * N, U = D::U, CL = D::CL, E1 = D::E > 0 ? D::E : 1;
+  const long long u = (long long)blockIdx.x * (DSS_THREADS / 32) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (u >= nunits) return;
+  const bool low = u >= nmain;
+  const long long v = low ? u - nmain : u;
+  long long t = low ? v / D::LOW : v / D::CHUNKS;
+  const int q = (int)(low ? v - t * D::LOW : v - t * D::CHUNKS);
+  if (low) { // the t-th low-face tile
+    const long long nxy = (long long)g.ntx * g.nty, nxz = (long long)g.ntx * (g.ntz - 1);
+    if (t >= nxy) {
+      long long r = t - nxy;
+      if (r < nxz) { // ty = 0, tz >= 1
+        t = (1 + r / g.ntx) * nxy + r % g.ntx;
+      } else { // tx = 0, ty, tz >= 1
+        r -= nxz;
+        t = (1 + r / (g.nty - 1)) * nxy + (1 + r % (g.nty - 1)) * g.ntx;
+      }
+    }
+  }
+  int cx, cy, cz;
+  cell_of(g, t, lane, cx, cy, cz);
+  if (cx >= g.nx || cy >= g.ny || cz >= g.nz) return; // padding lane (no warp-wide operation below)
+  const int lx = lane & 3, ly = (lane >> 2) & 3, lz = lane >> 4;
+  const long long tile_el = (long long)N3 * BL;
+  DssLane d;
+  d.h[0] = cx < g.nx - 1;
+  d.h[1] = cy < g.ny - 1;
+  d.h[2] = cz < g.nz - 1;
+  d.o[0] = lx < TX - 1 ? 1 - K * BL : tile_el - K * BL - (TX - 1);
+  d.o[1] = ly < TY - 1 ? TX - K * N * BL : g.ntx * tile_el - K * N * BL - TX * (TY - 1);
+  d.o[2] =
+      lz < TZ - 1 ? TX * TY - K * N2 * BL : (long long)g.ntx * g.nty * tile_el - K * N2 * BL - TX * TY * (TZ - 1);
+  d.mask = g.bc && !avg;
+  d.avg = avg;
+  T* y0 = y + t * tile_el + lane;
+  if (low) {
+    int i, j, k, r = q; // row q of those with a zero index: k = 0, then j = 0, then i = 0
+    if (r < N2) {
+      k = 0; j = r / N; i = r % N;
+    } else if ((r -= N2) < N * K) {
+      j = 0; k = 1 + r / N; i = r % N;
+    } else {
+      r -= N * K;
+      i = 0; j = 1 + r % K; k = 1 + r / K;
+    }
+    if ((i == 0 && cx > 0) || (j == 0 && cy > 0) || (k == 0 && cz > 0)) return; // not the lowest copy
+    T* p = y0 + (i + N * j + N2 * k) * BL;
+    switch ((i == K ? 1 : 0) | (j == K ? 2 : 0) | (k == K ? 4 : 0)) { // uniform
+      case 0: dss_rows<T, false, false, false, 1, 0>(p, d, 1, true); break;
+      case 1: dss_rows<T, true, false, false, 1, 0>(p, d, 1, true); break;
+      case 2: dss_rows<T, false, true, false, 1, 0>(p, d, 1, true); break;
+      case 3: dss_rows<T, true, true, false, 1, 0>(p, d, 1, true); break;
+      case 4: dss_rows<T, false, false, true, 1, 0>(p, d, 1, true); break;
+      case 5: dss_rows<T, true, false, true, 1, 0>(p, d, 1, true); break;
+      default: dss_rows<T, false, true, true, 1, 0>(p, d, 1, true); break; // one index is 0: never all three
+    }
+    return;
+  }
+  // rows with i, j, k >= 1 on a high face of the cell
+  if (q == 0) {
+    dss_rows<T, true, true, true, 1, 0>(y0 + (K + N * K + N2 * K) * BL, d, 1, false);
+    return;
+  }
+  // line: 0..2 the edges along x, y, z; then E lines on each of the z, y and x faces
+  const int line = (q - 1) / CL, first = 1 + ((q - 1) - line * CL) * U, count = min(U, K - first);
+  if (line < 3) {
+    if (line == 0) dss_rows<T, false, true, true, U, BL>(y0 + (first + N * K + N2 * K) * BL, d, count, false);
+    else if (line == 1) dss_rows<T, true, false, true, U, N * BL>(y0 + (K + N * first + N2 * K) * BL, d, count, false);
+    else dss_rows<T, true, true, false, U, N2 * BL>(y0 + (K + N * K + N2 * first) * BL, d, count, false);
+  } else {
+    const int f = (line - 3) / E1, m = 1 + (line - 3) - f * E1;
+    if (f == 0) dss_rows<T, false, false, true, U, BL>(y0 + (first + N * m + N2 * K) * BL, d, count, false);
+    else if (f == 1) dss_rows<T, false, true, false, U, BL>(y0 + (first + N * K + N2 * m) * BL, d, count, false);
+    else dss_rows<T, true, false, false, U, N * BL>(y0 + (K + N * first + N2 * m) * BL, d, count, false);
   }
 }
 
@@ -1729,30 +1795,14 @@ mf_status apply_batch_launch_n(const mf_operator* op0, int vk, const void* jobs_
   if (vk == VK_DD) return batch_launch_t<double, dd, N>(op0, v, jobs_dev, block0_dev, njobs, blocks, s);
   return batch_launch_t<double, double, N>(op0, v, jobs_dev, block0_dev, njobs, blocks, s);
 }
-// The row kernel from degree 2 (measured: k = 3, 92^3: 0.204 ms against 0.277 ms); degree 1,
-// whose rows hold a single local index, keeps the lexicographic one (0.159 against 0.179 ms).
-// MF_DSS_ROWS=0 selects the lexicographic kernel everywhere (same sums, bitwise).
-#ifndef MF_DSS_ROWS
-#define MF_DSS_ROWS 1
-#endif
 template <int N>
 static mf_status dss_mode(const mf_operator* op, int elem, void* y, int avg, cudaStream_t s) {
-  if (MF_DSS_ROWS && N > 2) {
-    const int cxb = (op->g.nx + 1 + DSS_ROW_THREADS - 1) / DSS_ROW_THREADS; // nx + 1 columns at i = 0
-    const long long NYn = (long long)op->g.ny * (N - 1) + 1, NZn = (long long)op->g.nz * (N - 1) + 1;
-    const dim3 grid((unsigned)((N - 1) * cxb), (unsigned)(NYn < DSS_ROWS_Y ? NYn : DSS_ROWS_Y),
-                    (unsigned)(NZn < 65535 ? NZn : 65535));
-    if (elem == 8)
-      dss_row_kernel<double, N><<<grid, DSS_ROW_THREADS, 0, s>>>(static_cast<double*>(y), op->g, avg, cxb);
-    else
-      dss_row_kernel<float, N><<<grid, DSS_ROW_THREADS, 0, s>>>(static_cast<float*>(y), op->g, avg, cxb);
-    return cuda_check(cudaGetLastError(), "dss launch");
-  }
-  const long long total = op->n_unique;
-  const int thr = 256;
-  const long long blocks = (total + thr - 1) / thr;
-  if (elem == 8) dss_kernel<double, N><<<(unsigned)blocks, thr, 0, s>>>(static_cast<double*>(y), op->g, avg);
-  else dss_kernel<float, N><<<(unsigned)blocks, thr, 0, s>>>(static_cast<float*>(y), op->g, avg);
+  const GridInfo& g = op->g;
+  const long long nlow = g.ntiles - (long long)(g.ntx - 1) * (g.nty - 1) * (g.ntz - 1);
+  const long long nmain = g.ntiles * DssCfg<N>::CHUNKS, units = nmain + nlow * DssCfg<N>::LOW;
+  const unsigned blocks = (unsigned)((units + DSS_THREADS / 32 - 1) / (DSS_THREADS / 32));
+  if (elem == 8) dss_kernel<double, N><<<blocks, DSS_THREADS, 0, s>>>(static_cast<double*>(y), g, avg, nmain, units);
+  else dss_kernel<float, N><<<blocks, DSS_THREADS, 0, s>>>(static_cast<float*>(y), g, avg, nmain, units);
   return cuda_check(cudaGetLastError(), "dss launch");
 }
 template <int N>
