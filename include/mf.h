@@ -107,9 +107,12 @@ mf_status mf_operator_info(const mf_operator* op, mf_info* info);
  * must outlive the operator. */
 mf_status mf_operator_setup(mf_operator* op, void* workspace_dev, size_t bytes, void* stream);
 
-/* Autotuner: times each launch configuration of the apply kernel (variant 0: n^2 x CB
- * threads per CTA, registers capped for two CTAs per SM; variant 1: half the cells per CTA,
- * capped for three; variant 2: half the cells per CTA, no register cap; variant 3, for
+/* Autotuner: times each launch configuration of the apply kernel (variant 0: the configuration
+ * measured fastest for the operator's degree, path and precision -- one thread per plane of a
+ * cell for MF_FP32 up to degree 5 (6 on Cartesian meshes) and MF_FP64 of degree 1 and 2, else one
+ * of the pencil configurations; variant 1: one thread per pencil, half of the base configuration's
+ * n^2 x CB threads per CTA, registers capped for three CTAs per SM; variant 2: half the cells per
+ * CTA, no register cap; variant 3, for
  * MF_FP64 operators on an axis-aligned affine mesh of degree 1..3 only: the tensor-core
  * apply, see MF_VARIANT_TENSOR; variants 4 and 5, for MF_FP64 (double-float) operators
  * only: see MF_VARIANT_SMALL_CTA and MF_VARIANT_OCCUPANCY) with `reps` applies of x_dev into
@@ -136,13 +139,13 @@ mf_status mf_operator_autotune(mf_operator* op, const void* x_dev, void* y_dev, 
  * per value.  A non-finite input value makes its cell's outputs NaN.  Needs
  * mf_operator_setup (the digit table lives in the operator workspace, at most 48 KB). */
 #define MF_VARIANT_TENSOR 3
-/* Half the cells per CTA of variant 0 (the B axis of the paper's block-size experiment,
- * Sec. 6; see mf_apply_split_block), with registers capped for 1.5x variant 0's resident
+/* Half the cells per CTA of the base pencil configuration (the B axis of the paper's block-size experiment,
+ * Sec. 6; see mf_apply_split_block), with registers capped for 1.5x its resident
  * threads per SM.  Double-float view of MF_FP64 operators; same per-thread arithmetic as
  * variants 0-2 (bitwise equal results). */
 #define MF_VARIANT_SMALL_CTA 4
-/* Variant 0's cells per CTA with registers capped for three resident CTAs per SM instead of
- * two.  Double-float view of MF_FP64 operators; bitwise equal results. */
+/* The base pencil configuration's cells per CTA with registers capped for three resident CTAs
+ * per SM instead of two.  Double-float view of MF_FP64 operators; bitwise equal results. */
 #define MF_VARIANT_OCCUPANCY 5
 /* Forces a launch variant (0, 1 or 2) for every precision view, or MF_VARIANT_TENSOR /
  * MF_VARIANT_SMALL_CTA / MF_VARIANT_OCCUPANCY for the double-float view of an MF_FP64
@@ -200,7 +203,8 @@ mf_status mf_dss_atomic(const mf_operator* op, void* y_dev, void* scratch_dev, s
 /* Block-size sweep (a measurement entry: the paper sweeps the cells per thread block B of
  * its volume kernel, Sec. 6): mf_apply_split with cells_per_cta = B in {4, 8, 16, 32} cells
  * per CTA -- divisors of the 32-cell layout tile -- instead of the launch variant's.
- * Registers are capped so that every B keeps launch variant 0's resident threads per SM.
+ * Registers are capped so that every B keeps the base pencil configuration's resident threads
+ * per SM.
  * Same result as mf_apply_split with launch variant 0 (the arithmetic of a cell does not
  * depend on B), no duplicate summation.  Built for degree 3 on every path with MF_FP64
  * (double-float) and MF_FP32 operators, and for the Cartesian path of MF_FP64 operators at
@@ -213,7 +217,7 @@ mf_status mf_apply_split_block(const mf_operator* op, int cells_per_cta, const v
 /* Stream twin of the apply kernel (a measurement entry: the paper times kernels that keep a
  * kernel's memory accesses and drop its arithmetic, Sec. 6, as the ceiling of its access
  * pattern).  One launch with the apply's grid and cells per CTA (the operator's launch
- * variant) and its global accesses: the cell-wise x tile of every CTA is read; for a curved
+ * variant; for variant 0 the base pencil configuration's) and its global accesses: the cell-wise x tile of every CTA is read; for a curved
  * mesh in an FP64 precision the per-point metric (6 words per point, 7 for Helmholtz, 8 bytes
  * each) is read as the apply streams it; y is written by x-pencils.  No contraction and no
  * duplicate summation.  y_dev receives a bit-copy of x_dev, not an operator result.

@@ -461,7 +461,7 @@ static std::string tune_key(int dev, const mf_operator* op, int vk) {
   std::string name = "unknown";
   if (cudaGetDeviceProperties(&prop, dev) == cudaSuccess) name = prop.name;
   char buf[160];
-  std::snprintf(buf, sizeof(buf), "|lib=4|n=%d|path=%d|kind=%d|view=%d|cells=2^%d", op->n, op->path, op->kind, vk,
+  std::snprintf(buf, sizeof(buf), "|lib=5|n=%d|path=%d|kind=%d|view=%d|cells=2^%d", op->n, op->path, op->kind, vk,
                 tune_size_class(op));
   return name + buf;
 }

@@ -133,7 +133,9 @@ __host__ __device__ __forceinline__ double f2d_bits(float f) {
 __host__ __device__ __forceinline__ double dd_to_double(dd a) { return f2d_bits(a.hi) + f2d_bits(a.lo); }
 
 // Two FP32 values of neighbouring cells processed by one thread (the FP32 apply): every
-// operation acts on both lanes; table coefficients stay scalar floats.
+// operation acts on both lanes; table coefficients stay scalar floats.  Products and sums that
+// are not an fma() are single rounded operations (no contraction), so that kernels of different
+// shape give bitwise equal results.
 struct __align__(8) f2 {
   float x, y;
   __host__ __device__ f2() {}
@@ -142,12 +144,12 @@ struct __align__(8) f2 {
 };
 __device__ __forceinline__ f2 fma(float c, f2 a, f2 b) { return f2(fmaf(c, a.x, b.x), fmaf(c, a.y, b.y)); }
 __device__ __forceinline__ f2 fma(f2 c, f2 a, f2 b) { return f2(fmaf(c.x, a.x, b.x), fmaf(c.y, a.y, b.y)); }
-__device__ __forceinline__ f2 mul0(float c, f2 a) { return f2(c * a.x, c * a.y); }
-__device__ __forceinline__ f2 mul0(f2 c, f2 a) { return f2(c.x * a.x, c.y * a.y); }
+__device__ __forceinline__ f2 mul0(float c, f2 a) { return f2(__fmul_rn(c, a.x), __fmul_rn(c, a.y)); }
+__device__ __forceinline__ f2 mul0(f2 c, f2 a) { return f2(__fmul_rn(c.x, a.x), __fmul_rn(c.y, a.y)); }
 __device__ __forceinline__ f2 finish(f2 a) { return a; }
-__device__ __forceinline__ f2 operator*(float c, f2 a) { return f2(c * a.x, c * a.y); }
-__device__ __forceinline__ f2 operator*(f2 c, f2 a) { return f2(c.x * a.x, c.y * a.y); }
-__device__ __forceinline__ f2 operator+(f2 a, f2 b) { return f2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ f2 operator*(float c, f2 a) { return mul0(c, a); }
+__device__ __forceinline__ f2 operator*(f2 c, f2 a) { return mul0(c, a); }
+__device__ __forceinline__ f2 operator+(f2 a, f2 b) { return f2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)); }
 __device__ __forceinline__ f2 operator-(f2 a) { return f2(-a.x, -a.y); }
 
 // Coefficient type of the 1D tables for a compute type, and cells per compute value.

@@ -117,9 +117,10 @@ struct ApplyJob {
   T mdet;                     // affine: mass_coeff * |det J|
   T gx, gy, gz, cmass;        // Cartesian: det/h_d^2 and mass_coeff * det
   // FP32 curved: the metric is computed per point from per-direction tables of
-  // sin(pi xh), cos(pi xh) at the Gauss points of every cell layer ([(nx+ny+nz)*N][2]).
+  // sin(pi xh), pi cos(pi xh) at the Gauss points of every cell layer ([(nx+ny+nz)*N][2]);
+  // ih: 1/h per direction, hdet: h_x h_y h_z.
   const float* gtab;
-  float amp, cm, h[3];
+  float amp, cm, ih[3], hdet;
   CgFuse<S> cg; // cg.st == nullptr: plain apply
   // L2 prefetch distance in tiles (about one wave of resident CTAs ahead; 0 = off): the first
   // CTA of tile t prefetches the input and geometry of tile t + pf_tiles; pf_geom = 1 only

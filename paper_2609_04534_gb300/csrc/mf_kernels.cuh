@@ -18,9 +18,10 @@ namespace mf {
 // Cells processed by one CTA of the apply kernels (a divisor of BL).  One thread owns one
 // pencil (a 1D line of n values) of one cell -- of two cells for f2 -- in every sweep, so a
 // CTA has n^2 * CB threads.
-// Launch configurations of the apply kernels, chosen per operator by the autotuner
-// (mf_operator_autotune): variant 0 = CB0 cells per CTA with registers capped for 2 resident
-// CTAs per SM; variant 1 = CB0/2 cells per CTA, capped for 3 resident CTAs per SM;
+// Launch configurations of the pencil kernels, chosen per operator by the autotuner
+// (mf_operator_autotune): base configuration Cfg 0 = CB0 cells per CTA with registers capped for 2
+// resident CTAs per SM (launch variant 0 is the fastest of these per degree and path, or a plane
+// kernel: see variant0 and mf_plane.cuh); variant 1 = CB0/2 cells per CTA, capped for 3 resident CTAs per SM;
 // variant 2 = CB0/2 cells per CTA with no register cap (high degrees spill under a cap);
 // variant 4 (double-float compute only) = CB0/2 cells per CTA, registers capped for 1.5x
 // variant 0's resident threads per SM; variant 5 (double-float only) = CB0 cells per CTA,
@@ -139,8 +140,8 @@ __device__ __forceinline__ T chain(const C* c, const T* x) {
   for (int i = 1; i < M; ++i) s = fma(c[i], x[i], s);
   return s;
 }
-__device__ __forceinline__ f2 add_lazy(f2 a, f2 b) { return f2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ f2 sub_lazy(f2 a, f2 b) { return f2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ f2 add_lazy(f2 a, f2 b) { return a + b; }
+__device__ __forceinline__ f2 sub_lazy(f2 a, f2 b) { return a + (-b); }
 
 // Even-odd 1D contraction of one pencil (see EoTab): the pencil folded into its sum and
 // difference halves, H (H + 1) products per half instead of n^2 in all.  ANTI: the matrix is
@@ -577,34 +578,66 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
   }
 }
 
-// The metric of the FP32 curved view at one Gauss point of one cell, computed from the sin
-// and cos of pi xh per direction: the map x = xh + amp s(xh) (1,1,1) has J = (I + u v^T) D
-// with u = amp (1,1,1), v = grad s, D = diag(h); Sherman-Morrison gives J^-1 = D^-1 (I - u v^T
-// / beta), beta = 1 + v.u, and J^-1 J^-T = D^-1 (I - (u v^T + v u^T)/beta + |v|^2 u u^T /
-// beta^2) D^-1.  g[0..5] = w |det J| J^-1 J^-T (xx, xy, xz, yy, yz, zz), g[6] = w |det J| c_m.
-template <typename S, typename T>
-__device__ __forceinline__ void curved_metric_f32(float sx, float cxv, float sy, float cyv, float sz, float czv,
-                                                  float wq, const ApplyJob<S, T>& a, float* g) {
-  const float pi = 3.14159265358979f;
-  const float v1 = pi * cxv * sy * sz, v2 = pi * sx * cyv * sz, v3 = pi * sx * sy * czv;
-  const float beta = fmaf(a.amp, v1 + v2 + v3, 1.0f);
-  const float ib = 1.0f / beta;
-  const float au = a.amp * ib;
-  const float c2 = au * au * (v1 * v1 + v2 * v2 + v3 * v3);
-  const float wd = wq * (a.h[0] * a.h[1] * a.h[2]) * fabsf(beta);
-  const float i0 = 1.0f / a.h[0], i1 = 1.0f / a.h[1], i2 = 1.0f / a.h[2];
-  g[0] = wd * i0 * i0 * (1.0f - 2.0f * au * v1 + c2);
-  g[1] = wd * i0 * i1 * (c2 - au * (v1 + v2));
-  g[2] = wd * i0 * i2 * (c2 - au * (v1 + v3));
-  g[3] = wd * i1 * i1 * (1.0f - 2.0f * au * v2 + c2);
-  g[4] = wd * i1 * i2 * (c2 - au * (v2 + v3));
-  g[5] = wd * i2 * i2 * (1.0f - 2.0f * au * v3 + c2);
-  g[6] = wd * a.cm;
+// 1 / b for b well inside the float range (here in [0.6, 1.4]): the hardware's approximation
+// (1 ulp) and one Newton-Raphson step, x (2 - b x); within 1 ulp of the division, whose range
+// handling costs several times as much (Q4 curved FP32 52^3, plane kernel: 0.110 -> 0.099 ms).
+// The pencil kernels of n = 7, 8 keep the division (n = 7: 0.162 against 0.174 ms, n = 8: 0.175
+// against 0.195 with the Newton step, which costs them registers).
+template <int N>
+__device__ __forceinline__ float metric_rcp(float b) {
+  if constexpr (N == 7 || N == 8) return __frcp_rn(b);
+  float x;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(b));
+  return fmaf(x, fmaf(-b, x, 1.0f), x);
 }
-template <typename T>
-__device__ __forceinline__ T pack_lanes(const float (*g)[7], int m) {
-  if constexpr (CellsPer<T>::value == 2) return T(g[0][m], g[1][m]);
-  else return T(g[0][m]);
+
+// Flux v = G d of the FP32 curved view at one Gauss point of one cell (d the reference
+// gradient), and m = w |det J| c_m, from the sin and pi cos of pi xh per direction: the map
+// x = xh + amp s(xh) (1,1,1) has J = (I + u v^T) D with u = amp (1,1,1), v = grad s, D = diag(h);
+// Sherman-Morrison gives J^-1 = D^-1 (I - u v^T / beta), beta = 1 + v.u, and J^-1 J^-T = D^-1
+// (I - (u v^T + v u^T)/beta + |v|^2 u u^T / beta^2) D^-1.  G is applied as it stands, one
+// rank-one term at a time (23 operations instead of 21 to form its six entries and 9 to apply
+// them).  Arguments: sx, pi cos x, and the products sy sz, pi cos y sz, sy pi cos z.  Every
+// operation is rounded as written (no contraction), see f2.
+template <int N, typename S, typename T>
+__device__ __forceinline__ void curved_flux_f32(float sx, float px, float syz, float pyz, float spz, float w,
+                                                const ApplyJob<S, T>& a, float d1, float d2, float d3, float* v,
+                                                float* m) {
+  const float v1 = __fmul_rn(px, syz), v2 = __fmul_rn(sx, pyz), v3 = __fmul_rn(sx, spz);
+  const float beta = fmaf(a.amp, __fadd_rn(__fadd_rn(v1, v2), v3), 1.0f);
+  const float au = __fmul_rn(a.amp, metric_rcp<N>(beta));
+  const float vv = fmaf(v3, v3, fmaf(v2, v2, __fmul_rn(v1, v1)));
+  const float c2 = __fmul_rn(__fmul_rn(au, au), vv);
+  const float wd = __fmul_rn(__fmul_rn(w, a.hdet), fabsf(beta));
+  const float e1 = __fmul_rn(a.ih[0], d1), e2 = __fmul_rn(a.ih[1], d2), e3 = __fmul_rn(a.ih[2], d3); // D^-1 d
+  const float s = __fadd_rn(__fadd_rn(e1, e2), e3), t = fmaf(v3, e3, fmaf(v2, e2, __fmul_rn(v1, e1)));
+  const float k = fmaf(c2, s, -__fmul_rn(au, t)), as = __fmul_rn(au, s);
+  v[0] = __fmul_rn(__fmul_rn(wd, a.ih[0]), fmaf(-as, v1, __fadd_rn(e1, k)));
+  v[1] = __fmul_rn(__fmul_rn(wd, a.ih[1]), fmaf(-as, v2, __fadd_rn(e2, k)));
+  v[2] = __fmul_rn(__fmul_rn(wd, a.ih[2]), fmaf(-as, v3, __fadd_rn(e3, k)));
+  *m = __fmul_rn(wd, a.cm);
+}
+// the same for a value (a pair of x-neighbours: sx, px per cell)
+template <int N, typename S, typename T>
+__device__ __forceinline__ void curved_flux(const float (&sx)[2], const float (&px)[2], float syz, float pyz, float spz,
+                                            float w, const ApplyJob<S, T>& a, T d1, T d2, T d3, T& v1, T& v2, T& v3,
+                                            T& m) {
+  float v[3], mm;
+  if constexpr (CellsPer<T>::value == 2) {
+    float u[3], mu;
+    curved_flux_f32<N>(sx[0], px[0], syz, pyz, spz, w, a, d1.x, d2.x, d3.x, v, &mm);
+    curved_flux_f32<N>(sx[1], px[1], syz, pyz, spz, w, a, d1.y, d2.y, d3.y, u, &mu);
+    v1 = T(v[0], u[0]);
+    v2 = T(v[1], u[1]);
+    v3 = T(v[2], u[2]);
+    m = T(mm, mu);
+  } else if constexpr (IsF32<T>::value) {
+    curved_flux_f32<N>(sx[0], px[0], syz, pyz, spz, w, a, d1, d2, d3, v, &mm);
+    v1 = v[0];
+    v2 = v[1];
+    v3 = v[2];
+    m = mm;
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -683,11 +716,11 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
   const long long gbase = (t * NC * (long long)N3) * BL + lane0 + c * CellsPer<T>::value;
   const bool fuse = a.cg.st != nullptr;
   T pap = T(0);
-  // FP32 curved: sin / cos of pi xh at this thread's x and y points and at every z point of
+  // FP32 curved: sin and pi cos of pi xh at this thread's x and y points and at every z point of
   // the cell's layer, loaded before the point loop (per cell of the value: the cells of a
   // pair are x-neighbours, so only the x tables differ)
   constexpr int CPL = CellsPer<T>::value;
-  float sx[CPL], cxv[CPL], sy = 0.f, cyv = 0.f, szq[N], czq[N];
+  float sx[2], px[2], sy = 0.f, py = 0.f, szq[N], pzq[N];
   if constexpr (CURVED && IsF32<T>::value) {
     int ccx, ccy, ccz;
     cell_of(a.g, t, lane0 + c * CPL, ccx, ccy, ccz);
@@ -697,46 +730,43 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     for (int j = 0; j < CPL; ++j) {
       const float* tx = a.gtab + 2 * (min(ccx + j, a.g.nx - 1) * N + pa);
       sx[j] = tx[0];
-      cxv[j] = tx[1];
+      px[j] = tx[1];
     }
     const float* ty = a.gtab + 2 * ((a.g.nx + ccy) * N + pb);
     const float* tz = a.gtab + 2 * ((a.g.nx + a.g.ny + ccz) * N);
-    sy = ty[0]; cyv = ty[1];
+    sy = ty[0]; py = ty[1];
 #pragma unroll
-    for (int q = 0; q < N; ++q) { szq[q] = tz[2 * q]; czq[q] = tz[2 * q + 1]; }
+    for (int q = 0; q < N; ++q) { szq[q] = tz[2 * q]; pzq[q] = tz[2 * q + 1]; }
   }
 #pragma unroll
   for (int q = 0; q < N; ++q) {
     const int l = pa + N * pb + N2 * q;
-    const T d1 = buf0[l * CB + c], d2 = buf2[l * CB + c];
-    T g0, g1, g2, g3, g4, g5, m = T(0);
+    const T d1 = buf0[l * CB + c], d2 = buf2[l * CB + c], d3q = d3[q];
+    T v1, v2, v3, m = T(0);
     if constexpr (CURVED && IsF32<T>::value) {
-      float gg[CPL][7];
-#pragma unroll
-      for (int j = 0; j < CPL; ++j)
-        curved_metric_f32(sx[j], cxv[j], sy, cyv, szq[q], czq[q], tab.W[pa] * tab.W[pb] * tab.W[q], a, gg[j]);
-      g0 = pack_lanes<T>(gg, 0); g1 = pack_lanes<T>(gg, 1); g2 = pack_lanes<T>(gg, 2);
-      g3 = pack_lanes<T>(gg, 3); g4 = pack_lanes<T>(gg, 4); g5 = pack_lanes<T>(gg, 5);
-      if (HELM) m = pack_lanes<T>(gg, 6);
-    } else if (CURVED) {
-      const T* gp = a.geom + gbase + (long long)l * BL;
-      g0 = gp[0];
-      g1 = gp[(long long)1 * N3 * BL];
-      g2 = gp[(long long)2 * N3 * BL];
-      g3 = gp[(long long)3 * N3 * BL];
-      g4 = gp[(long long)4 * N3 * BL];
-      g5 = gp[(long long)5 * N3 * BL];
-      if (HELM) m = gp[(long long)6 * N3 * BL];
+      curved_flux<N>(sx, px, __fmul_rn(sy, szq[q]), __fmul_rn(py, szq[q]), __fmul_rn(sy, pzq[q]),
+                  tab.W[pa] * tab.W[pb] * tab.W[q], a, d1, d2, d3q, v1, v2, v3, m);
     } else {
-      const auto w = tab.W[pa] * tab.W[pb] * tab.W[q];
-      g0 = w * a.G[0]; g1 = w * a.G[1]; g2 = w * a.G[2];
-      g3 = w * a.G[3]; g4 = w * a.G[4]; g5 = w * a.G[5];
-      if (HELM) m = w * a.mdet;
+      T g0, g1, g2, g3, g4, g5;
+      if (CURVED) {
+        const T* gp = a.geom + gbase + (long long)l * BL;
+        g0 = gp[0];
+        g1 = gp[(long long)1 * N3 * BL];
+        g2 = gp[(long long)2 * N3 * BL];
+        g3 = gp[(long long)3 * N3 * BL];
+        g4 = gp[(long long)4 * N3 * BL];
+        g5 = gp[(long long)5 * N3 * BL];
+        if (HELM) m = gp[(long long)6 * N3 * BL];
+      } else {
+        const auto w = tab.W[pa] * tab.W[pb] * tab.W[q];
+        g0 = w * a.G[0]; g1 = w * a.G[1]; g2 = w * a.G[2];
+        g3 = w * a.G[3]; g4 = w * a.G[4]; g5 = w * a.G[5];
+        if (HELM) m = w * a.mdet;
+      }
+      v1 = finish(fma(g0, d1, fma(g1, d2, mul0(g2, d3q))));
+      v2 = finish(fma(g1, d1, fma(g3, d2, mul0(g4, d3q))));
+      v3 = finish(fma(g2, d1, fma(g4, d2, mul0(g5, d3q))));
     }
-    const T d3q = d3[q];
-    const T v1 = finish(fma(g0, d1, fma(g1, d2, mul0(g2, d3q))));
-    const T v2 = finish(fma(g1, d1, fma(g3, d2, mul0(g4, d3q))));
-    const T v3 = finish(fma(g2, d1, fma(g4, d2, mul0(g5, d3q))));
     buf0[l * CB + c] = v1;
     buf2[l * CB + c] = v2;
     d3[q] = v3;
@@ -762,17 +792,16 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     for (int j = 0; j < N; ++j) buf2[(pa + N * j + N2 * pb) * CB + c] = out[j];
   }
   __syncthreads();
-  // t = Dc^T_x v1 + Dc^T_y v2 + Dc^T_z v3 (+ m u) at points (pa, pb, q), then S^T along z
+  // t = Dc^T_x v1 (+ m u) + Dc^T_y v2 + Dc^T_z v3 at points (pa, pb, q), then S^T along z
   {
     T tq[N];
     Fold<T, N, true>(d3).apply(tab.eDt, tq); // Dc^T_z v3 along this pencil
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       const int l = pa + N * pb + N2 * q;
-      T s = add_lazy(buf1[l * CB + c], buf2[l * CB + c]);
-      s = add_lazy(s, tq[q]);
+      T s = buf1[l * CB + c];
       if (HELM) s = add_lazy(s, U[q]);
-      tq[q] = finish(s);
+      tq[q] = finish(add_lazy(add_lazy(s, buf2[l * CB + c]), tq[q]));
     }
     T out[N];
     Fold<T, N, false>(tq).apply(tab.eSt, out);
@@ -805,6 +834,12 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
   }
 }
 
+} // namespace mf
+
+#include "mf_plane.cuh"
+
+namespace mf {
+
 // Kernels: one operator per launch (CTA b = cells (b % GPT) * CB .. of tile b / GPT), or a
 // batch of operators of one degree (see ApplyBatch): the CTA finds its job by binary search
 // over the block offsets and copies the job's description into shared memory.
@@ -827,6 +862,15 @@ template <typename S, typename T, int N, int CB, int MINB, bool CURVED, bool HEL
 __global__ void __launch_bounds__(N * N * CB, MINB) apply_general(ApplyArgs<S, T, N> A) {
   constexpr int CC = CB * CellsPer<T>::value, GPT = BL / CC;
   general_body<S, T, N, CB, CURVED, HELM>(A.j, A.tab, blockIdx.x / GPT, (blockIdx.x % GPT) * CC, blockIdx.x);
+}
+
+template <typename S, typename T, int N, bool HELM>
+__global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_C) apply_cartesian_plane(ApplyArgs<S, T, N> A) {
+  cartesian_plane<S, T, N, HELM>(A.j, A.tab, blockIdx.x);
+}
+template <typename S, typename T, int N, bool CURVED, bool HELM>
+__global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_G) apply_general_plane(ApplyArgs<S, T, N> A) {
+  general_plane<S, T, N, CURVED, HELM>(A.j, A.tab, blockIdx.x);
 }
 
 // The batched apply is one persistent launch: as many CTAs as fit the GPU at once, each
@@ -886,6 +930,31 @@ __global__ void __launch_bounds__(N * N * CB, MINB) apply_general_batch(ApplyBat
   }
 }
 
+template <typename S, typename T, int N, bool HELM>
+__global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_C)
+    apply_cartesian_plane_batch(ApplyBatch<S, T, N> B) {
+  __shared__ __align__(16) ApplyJob<S, T> sj;
+  __shared__ int jheld;
+  if (threadIdx.x == 0) jheld = -1;
+  for (long long u = blockIdx.x; u < B.nunits; u += gridDim.x) {
+    const long long b = batch_unit(B.jobs, B.block0, B.njobs, u, sj, jheld);
+    cartesian_plane<S, T, N, HELM>(sj, B.tab, b);
+    __syncthreads();
+  }
+}
+template <typename S, typename T, int N, bool CURVED, bool HELM>
+__global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_G)
+    apply_general_plane_batch(ApplyBatch<S, T, N> B) {
+  __shared__ __align__(16) ApplyJob<S, T> sj;
+  __shared__ int jheld;
+  if (threadIdx.x == 0) jheld = -1;
+  for (long long u = blockIdx.x; u < B.nunits; u += gridDim.x) {
+    const long long b = batch_unit(B.jobs, B.block0, B.njobs, u, sj, jheld);
+    general_plane<S, T, N, CURVED, HELM>(sj, B.tab, b);
+    __syncthreads();
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // Duplicate summation y <- G G^T y (Sec. 4: embedding G and assembly G^T) in the canonical
 // order of the dimension-split sweeps of Sec. 3: the copies of a node are summed pairwise
@@ -917,8 +986,8 @@ struct DssCfg {
   // vertex.  A warp takes one chunk of U rows along a line (U loads in flight per copy and
   // lane), CL chunks per line, so that a copy's address is one pointer plus constant offsets.
   // (A loop over chunks made the compiler keep every kind's pointers: 160 registers.)
-  static constexpr int U = E < 1 ? 1 : (E <= 4 ? E : (E + 1) / 2), CL = (E + U - 1) / U;
-  static constexpr int CHUNKS = 1 + 3 * CL + 3 * CL * E;
+  static constexpr int U = E < 1 ? 1 : (E <= 4 ? E : (E + 1) / 2), CL = E < 1 ? 1 : (E + U - 1) / U;
+  static constexpr int CHUNKS = E < 1 ? 1 : 1 + 3 * CL + 3 * CL * E;
   static constexpr int LOW = N * N * N - K * K * K; // rows with a zero index
 };
 
@@ -1211,7 +1280,7 @@ struct GeomArgsQ {
   double qx[MAXN];
 };
 
-// FP32 curved view: sin(pi xh) and cos(pi xh) at the Gauss points of every cell layer, per
+// FP32 curved view: sin(pi xh) and pi cos(pi xh) at the Gauss points of every cell layer, per
 // direction ([(nx+ny+nz) * N][2] floats), computed in FP64 once at set-up.
 template <int N>
 __global__ void geom_table_kernel(float* tab, GridInfo g, GeomArgsQ q) {
@@ -1223,7 +1292,7 @@ __global__ void geom_table_kernel(float* tab, GridInfo g, GeomArgsQ q) {
   double sp, cp;
   sincospi((c + q.qx[qq]) / nd, &sp, &cp);
   tab[2 * e] = (float)sp;
-  tab[2 * e + 1] = (float)cp;
+  tab[2 * e + 1] = (float)(3.141592653589793238462643383279502884 * cp);
 }
 
 template <typename T>
@@ -1300,7 +1369,7 @@ struct DiagArgs {
   float S[MAXN * MAXN], D[MAXN * MAXN], W[MAXN];
   int curved;
   float G[6], mdet;                 // affine metric (w-free) and mass * det
-  const float* gtab;                // curved: sin / cos of pi xh per cell layer and direction
+  const float* gtab;                // curved: sin and pi cos of pi xh per cell layer and direction
   float amp, cm, h[3];
 };
 
@@ -1322,7 +1391,6 @@ __global__ void diag_kernel(float* __restrict__ dg, DiagArgs a) {
   const float* tx = a.gtab + 2 * (cx * N);
   const float* ty = a.gtab + 2 * ((a.g.nx + cy) * N);
   const float* tz = a.gtab + 2 * ((a.g.nx + a.g.ny + cz) * N);
-  const float pi = 3.14159265358979f;
   float acc = 0.0f;
   for (int qz = 0; qz < N; ++qz) {
     const float Sz = a.S[qz * MAXN + iz], Dz = a.D[qz * MAXN + iz];
@@ -1338,7 +1406,7 @@ __global__ void diag_kernel(float* __restrict__ dg, DiagArgs a) {
           // the metric of the curved map (same closed form as the FP32 apply)
           const float sx = tx[2 * qx], cxv = tx[2 * qx + 1], sy = ty[2 * qy], cyv = ty[2 * qy + 1];
           const float sz = tz[2 * qz], czv = tz[2 * qz + 1];
-          const float v1 = pi * cxv * sy * sz, v2 = pi * sx * cyv * sz, v3 = pi * sx * sy * czv;
+          const float v1 = cxv * sy * sz, v2 = sx * cyv * sz, v3 = sx * sy * czv;
           const float beta = fmaf(a.amp, v1 + v2 + v3, 1.0f);
           const float au = a.amp / beta;
           const float c2 = au * au * (v1 * v1 + v2 * v2 + v3 * v3);
@@ -1451,9 +1519,10 @@ static void fill_job(const mf_operator* op, ApplyJob<S, T>& a) {
   a.gtab = static_cast<const float*>(op->v32.geom);
   a.amp = (float)op->mesh.amp;
   a.cm = (float)(op->kind == MF_HELMHOLTZ ? op->mass : 0.0);
-  a.h[0] = 1.0f / op->g.nx;
-  a.h[1] = 1.0f / op->g.ny;
-  a.h[2] = 1.0f / op->g.nz;
+  a.ih[0] = (float)op->g.nx;
+  a.ih[1] = (float)op->g.ny;
+  a.ih[2] = (float)op->g.nz;
+  a.hdet = (float)(1.0 / ((double)op->g.nx * op->g.ny * op->g.nz));
   a.cg = CgFuse<S>{};
   a.pf_tiles = 0;
   a.pf_geom = 0;
@@ -1573,10 +1642,82 @@ struct BCfg {
 template <int N, int B>
 constexpr bool block_fits() { return N * N * B <= 1024 && N * N * B >= 32; }
 
-// C: the launch configuration (cells per CTA CB * CPL, MINB resident CTAs, NT threads)
+// What a launch needs besides its arguments: the kernel, its CTA and grid.  K: the one-operator
+// kernel's type or the batched one's.
+template <typename K>
+struct Shape {
+  K kernel = nullptr;
+  int threads = 0, ctas_per_tile = 1, tiles_per_cta = 1;
+  size_t smem = 0;
+  long long blocks(long long ntiles) const {
+    return (ntiles * ctas_per_tile + tiles_per_cta - 1) / tiles_per_cta;
+  }
+};
+// C: the pencil kernels' launch configuration (cells per CTA CB * CPL, MINB resident CTAs, NT threads)
 template <typename S, typename T, int N, typename C>
-static mf_status apply_split_c(const mf_operator* op, const void* x, void* y, const void* geom, const CgFuse<S>& cg,
-                               long long* nblocks, cudaStream_t s) {
+static mf_status pencil_shape(const mf_operator* op, Shape<void (*)(ApplyArgs<S, T, N>)>& h) {
+  const bool helm = op->kind == MF_HELMHOLTZ;
+  // buffers of n^3 values per cell: Cartesian 1 (fast-diagonalised) or 2, general 3
+  h.smem = (op->path == PATH_CARTESIAN ? (MF_CART_FD ? 1 : 2) : 3) * sizeof(T) * N * N * N * C::CB;
+  h.threads = C::NT;
+  h.ctas_per_tile = BL / (C::CB * C::CPL);
+  if (op->path == PATH_CARTESIAN) {
+    h.kernel = helm ? apply_cartesian<S, T, N, C::CB, C::MINB, true> : apply_cartesian<S, T, N, C::CB, C::MINB, false>;
+  } else if constexpr (C::GENERAL) {
+    if (op->path == PATH_AFFINE)
+      h.kernel = helm ? apply_general<S, T, N, C::CB, C::MINB, false, true>
+                      : apply_general<S, T, N, C::CB, C::MINB, false, false>;
+    else
+      h.kernel =
+          helm ? apply_general<S, T, N, C::CB, C::MINB, true, true> : apply_general<S, T, N, C::CB, C::MINB, true, false>;
+  } else {
+    return set_error(MF_ERR_UNSUPPORTED, "block-size sweep: built for the Cartesian path at this degree");
+  }
+  return MF_OK;
+}
+// The plane kernels, where they are built (false elsewhere)
+template <typename T, int N>
+static bool use_plane(const mf_operator* op) {
+  return op->path == PATH_CARTESIAN ? UsePlane<T, N, PATH_CARTESIAN>::value
+                                    : (op->path == PATH_AFFINE ? UsePlane<T, N, PATH_AFFINE>::value
+                                                               : UsePlane<T, N, PATH_CURVED>::value);
+}
+// The pencil configuration that launch variant 0 stands for where it is not a plane kernel: the
+// fastest measured on one GB300 per degree and path, for double-float (split apply, ms, the
+// configuration of Cfg 0 -> the chosen one; ~17M DoFs).  Cartesian: Q3 0.256 -> 0.181, Q4 0.311 ->
+// 0.228, Q5 0.291 -> 0.224, Q6 0.387 -> 0.315, Q7 0.379 -> 0.350, Q8 0.507 -> 0.428.  Affine: Q3
+// 0.457 -> 0.384, Q4 0.560 -> 0.468, Q6 0.766 -> 0.687, the others stay.  Curved: Q2 0.515 ->
+// 0.411, Q3 0.438 -> 0.419, Q5 0.646 -> 0.623, Q6 (Laplace) 0.771 -> 0.734, the others stay.
+template <typename T, int N>
+static int variant0(const mf_operator* op) {
+  if (!std::is_same<T, dd>::value) return 0;
+  if (op->path == PATH_CARTESIAN) return N == 7 || N == 9 ? MF_VARIANT_OCCUPANCY : (N >= 4 ? MF_VARIANT_SMALL_CTA : 0);
+  if (op->path == PATH_AFFINE) return N == 4 || N == 5 || N == 7 ? MF_VARIANT_OCCUPANCY : 0;
+  if (N == 3) return MF_VARIANT_SMALL_CTA;
+  if (N == 4 || N == 6) return 1;
+  return N == 7 && op->kind == MF_LAPLACE ? MF_VARIANT_OCCUPANCY : 0;
+}
+template <typename S, typename T, int N>
+static void plane_shape(const mf_operator* op, Shape<void (*)(ApplyArgs<S, T, N>)>& h) {
+  using P = PlaneCfg<T, N>;
+  const bool helm = op->kind == MF_HELMHOLTZ;
+  h.threads = P::NT;
+  h.tiles_per_cta = P::TPC;
+  h.smem = (op->path == PATH_CARTESIAN ? 1 : 2) * sizeof(T) * N * N * N * P::CB;
+  if constexpr (UsePlane<T, N, PATH_CARTESIAN>::value)
+    if (op->path == PATH_CARTESIAN)
+      h.kernel = helm ? apply_cartesian_plane<S, T, N, true> : apply_cartesian_plane<S, T, N, false>;
+  if constexpr (UsePlane<T, N, PATH_AFFINE>::value)
+    if (op->path == PATH_AFFINE)
+      h.kernel = helm ? apply_general_plane<S, T, N, false, true> : apply_general_plane<S, T, N, false, false>;
+  if constexpr (UsePlane<T, N, PATH_CURVED>::value)
+    if (op->path == PATH_CURVED)
+      h.kernel = helm ? apply_general_plane<S, T, N, true, true> : apply_general_plane<S, T, N, true, false>;
+}
+
+template <typename S, typename T, int N>
+static mf_status apply_launch(const mf_operator* op, const Shape<void (*)(ApplyArgs<S, T, N>)>& h, const void* x,
+                              void* y, const void* geom, const CgFuse<S>& cg, long long* nblocks, cudaStream_t s) {
   ApplyArgs<S, T, N> a;
   fill_job<S, T>(op, a.j);
   fill_tab<typename CoefOf<T>::type, N>(op, a.tab);
@@ -1584,39 +1725,38 @@ static mf_status apply_split_c(const mf_operator* op, const void* x, void* y, co
   a.j.x = static_cast<const S*>(x);
   a.j.y = static_cast<S*>(y);
   a.j.geom = static_cast<const T*>(geom);
-  const bool helm = op->kind == MF_HELMHOLTZ;
-  // buffers of n^3 values per cell: Cartesian 1 (fast-diagonalised) or 2, general 3
-  const size_t smem = (op->path == PATH_CARTESIAN ? (MF_CART_FD ? 1 : 2) : 3) * sizeof(T) * N * N * N * C::CB;
-  const long long blocks = op->g.ntiles * (BL / (C::CB * C::CPL));
+  const long long blocks = h.blocks(op->g.ntiles);
   if (nblocks) *nblocks = blocks;
   if (blocks <= 0) return MF_OK;
-  void (*k)(ApplyArgs<S, T, N>) = nullptr;
-  if (op->path == PATH_CARTESIAN) {
-    k = helm ? apply_cartesian<S, T, N, C::CB, C::MINB, true> : apply_cartesian<S, T, N, C::CB, C::MINB, false>;
-  } else if constexpr (C::GENERAL) {
-    if (op->path == PATH_AFFINE)
-      k = helm ? apply_general<S, T, N, C::CB, C::MINB, false, true>
-               : apply_general<S, T, N, C::CB, C::MINB, false, false>;
-    else
-      k = helm ? apply_general<S, T, N, C::CB, C::MINB, true, true> : apply_general<S, T, N, C::CB, C::MINB, true, false>;
-  } else {
-    return set_error(MF_ERR_UNSUPPORTED, "block-size sweep: built for the Cartesian path at this degree");
-  }
-  if (smem > 227 * 1024) return set_error(MF_ERR_UNSUPPORTED, "apply variant needs %zu bytes of shared memory", smem);
+  if (h.smem > 227 * 1024)
+    return set_error(MF_ERR_UNSUPPORTED, "apply variant needs %zu bytes of shared memory", h.smem);
   // the kernels also hold static shared memory (the CG partial's park, NT doubles, and a few
   // bytes of the compiler's), and static + dynamic above 48 KB needs the opt-in
-  if (smem + sizeof(double) * C::NT + 1024 > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (h.smem + sizeof(double) * h.threads + 1024 > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(h.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
     if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(apply)");
   }
-  a.j.pf_tiles = prefetch_distance_tiles((const void*)k, C::NT, smem, BL / (C::CB * C::CPL));
+  a.j.pf_tiles = prefetch_distance_tiles((const void*)h.kernel, h.threads, h.smem, h.ctas_per_tile) * h.tiles_per_cta;
   a.j.pf_geom = (op->path == PATH_CURVED && !IsF32<T>::value) ? 1 : 0;
-  k<<<(unsigned)blocks, C::NT, smem, s>>>(a);
+  h.kernel<<<(unsigned)blocks, h.threads, h.smem, s>>>(a);
   return cuda_check(cudaGetLastError(), "apply launch");
+}
+template <typename S, typename T, int N, typename C>
+static mf_status apply_split_c(const mf_operator* op, const void* x, void* y, const void* geom, const CgFuse<S>& cg,
+                               long long* nblocks, cudaStream_t s) {
+  Shape<void (*)(ApplyArgs<S, T, N>)> h;
+  mf_status st = pencil_shape<S, T, N, C>(op, h);
+  if (st) return st;
+  return apply_launch<S, T, N>(op, h, x, y, geom, cg, nblocks, s);
 }
 template <typename S, typename T, int N, int V>
 static mf_status apply_split_v(const mf_operator* op, const void* x, void* y, const void* geom, const CgFuse<S>& cg,
                                long long* nblocks, cudaStream_t s) {
+  if (V == 0 && use_plane<T, N>(op)) {
+    Shape<void (*)(ApplyArgs<S, T, N>)> h;
+    plane_shape<S, T, N>(op, h);
+    return apply_launch<S, T, N>(op, h, x, y, geom, cg, nblocks, s);
+  }
   return apply_split_c<S, T, N, Cfg<T, N, V>>(op, x, y, geom, cg, nblocks, s);
 }
 
@@ -1654,6 +1794,7 @@ mf_status apply_block_n(const mf_operator* op, int vk, int cells, const void* x,
 template <typename S, typename T, int N>
 static mf_status apply_split_t(const mf_operator* op, int variant, const void* x, void* y, const void* geom,
                                const CgFuse<S>& cg, long long* nblocks, cudaStream_t s) {
+  if (variant == 0 && !use_plane<T, N>(op)) variant = variant0<T, N>(op);
   if (variant == 1) return apply_split_v<S, T, N, 1>(op, x, y, geom, cg, nblocks, s);
   if (variant == 2) return apply_split_v<S, T, N, 2>(op, x, y, geom, cg, nblocks, s);
   if constexpr (std::is_same<T, dd>::value) {
@@ -1715,7 +1856,8 @@ static mf_status batch_fill_v(const BatchMember* m, int n, int vk, void* jobs_ho
     a.y = static_cast<S*>(m[i].q);
     a.geom = static_cast<const T*>(vk == VK_F32 ? op->v32.geom : op->v64.geom);
     block0_host[i] = b;
-    b += op->g.ntiles * (BL / (C::CB * C::CPL));
+    b += V == 0 && use_plane<T, N>(op) ? PlaneCfg<T, N>::blocks(op->g.ntiles)
+                                       : op->g.ntiles * (BL / (C::CB * C::CPL));
   }
   block0_host[n] = b;
   return MF_OK;
@@ -1731,31 +1873,52 @@ static mf_status batch_launch_v(const mf_operator* op0, const void* jobs_dev, co
   B.block0 = block0_dev;
   B.njobs = njobs;
   const bool helm = op0->kind == MF_HELMHOLTZ;
-  const size_t smem = (op0->path == PATH_CARTESIAN ? (MF_CART_FD ? 1 : 2) : 3) * sizeof(T) * N * N * N * C::CB;
   if (blocks <= 0 || njobs <= 0) return MF_OK;
-  void (*k)(ApplyBatch<S, T, N>) = nullptr;
-  if (op0->path == PATH_CARTESIAN)
-    k = helm ? apply_cartesian_batch<S, T, N, C::CB, C::MINB, true> : apply_cartesian_batch<S, T, N, C::CB, C::MINB, false>;
-  else if (op0->path == PATH_AFFINE)
-    k = helm ? apply_general_batch<S, T, N, C::CB, C::MINB, false, true>
-             : apply_general_batch<S, T, N, C::CB, C::MINB, false, false>;
-  else
-    k = helm ? apply_general_batch<S, T, N, C::CB, C::MINB, true, true>
-             : apply_general_batch<S, T, N, C::CB, C::MINB, true, false>;
-  if (smem > 227 * 1024) return set_error(MF_ERR_UNSUPPORTED, "apply variant needs %zu bytes of shared memory", smem);
-  if (smem + sizeof(double) * C::NT + sizeof(ApplyJob<S, T>) + 1024 > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  Shape<void (*)(ApplyBatch<S, T, N>)> h;
+  const bool plane = V == 0 && use_plane<T, N>(op0);
+  if (plane) {
+    using P = PlaneCfg<T, N>;
+    h.threads = P::NT;
+    h.smem = (op0->path == PATH_CARTESIAN ? 1 : 2) * sizeof(T) * N * N * N * P::CB;
+    if constexpr (V == 0 && UsePlane<T, N, PATH_CARTESIAN>::value)
+      if (op0->path == PATH_CARTESIAN)
+        h.kernel = helm ? apply_cartesian_plane_batch<S, T, N, true> : apply_cartesian_plane_batch<S, T, N, false>;
+    if constexpr (V == 0 && UsePlane<T, N, PATH_AFFINE>::value)
+      if (op0->path == PATH_AFFINE)
+        h.kernel =
+            helm ? apply_general_plane_batch<S, T, N, false, true> : apply_general_plane_batch<S, T, N, false, false>;
+    if constexpr (V == 0 && UsePlane<T, N, PATH_CURVED>::value)
+      if (op0->path == PATH_CURVED)
+        h.kernel = helm ? apply_general_plane_batch<S, T, N, true, true> : apply_general_plane_batch<S, T, N, true, false>;
+  } else {
+    h.threads = C::NT;
+    h.smem = (op0->path == PATH_CARTESIAN ? (MF_CART_FD ? 1 : 2) : 3) * sizeof(T) * N * N * N * C::CB;
+    if (op0->path == PATH_CARTESIAN)
+      h.kernel =
+          helm ? apply_cartesian_batch<S, T, N, C::CB, C::MINB, true> : apply_cartesian_batch<S, T, N, C::CB, C::MINB, false>;
+    else if (op0->path == PATH_AFFINE)
+      h.kernel = helm ? apply_general_batch<S, T, N, C::CB, C::MINB, false, true>
+                      : apply_general_batch<S, T, N, C::CB, C::MINB, false, false>;
+    else
+      h.kernel = helm ? apply_general_batch<S, T, N, C::CB, C::MINB, true, true>
+                      : apply_general_batch<S, T, N, C::CB, C::MINB, true, false>;
+  }
+  if (h.smem > 227 * 1024)
+    return set_error(MF_ERR_UNSUPPORTED, "apply variant needs %zu bytes of shared memory", h.smem);
+  if (h.smem + sizeof(double) * h.threads + sizeof(ApplyJob<S, T>) + 1024 > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(h.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
     if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(batched apply)");
   }
   // one persistent launch: the CTAs resident on the GPU at once, looping over the units
   B.nunits = blocks;
-  const long long grid = std::min<long long>(blocks, resident_ctas((const void*)k, C::NT, smem));
-  k<<<(unsigned)grid, C::NT, smem, s>>>(B);
+  const long long grid = std::min<long long>(blocks, resident_ctas((const void*)h.kernel, h.threads, h.smem));
+  h.kernel<<<(unsigned)grid, h.threads, h.smem, s>>>(B);
   return cuda_check(cudaGetLastError(), "batched apply launch");
 }
 
 template <typename S, typename T, int N>
 static mf_status batch_fill_t(const BatchMember* m, int n, int vk, int variant, void* jobs_host, long long* block0_host) {
+  if (variant == 0 && !use_plane<T, N>(m[0].op)) variant = variant0<T, N>(m[0].op);
   if (variant == 1) return batch_fill_v<S, T, N, 1>(m, n, vk, jobs_host, block0_host);
   if (variant == 2) return batch_fill_v<S, T, N, 2>(m, n, vk, jobs_host, block0_host);
   if constexpr (std::is_same<T, dd>::value) {
@@ -1767,6 +1930,7 @@ static mf_status batch_fill_t(const BatchMember* m, int n, int vk, int variant, 
 template <typename S, typename T, int N>
 static mf_status batch_launch_t(const mf_operator* op0, int variant, const void* jobs_dev, const long long* block0_dev,
                                 int njobs, long long blocks, cudaStream_t s) {
+  if (variant == 0 && !use_plane<T, N>(op0)) variant = variant0<T, N>(op0);
   if (variant == 1) return batch_launch_v<S, T, N, 1>(op0, jobs_dev, block0_dev, njobs, blocks, s);
   if (variant == 2) return batch_launch_v<S, T, N, 2>(op0, jobs_dev, block0_dev, njobs, blocks, s);
   if constexpr (std::is_same<T, dd>::value) {
