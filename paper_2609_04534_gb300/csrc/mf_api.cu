@@ -49,6 +49,7 @@ mf_status cuda_check(cudaError_t e, const char* what) {
 mf_status launch_apply_split(const mf_operator* op, int elem, const void* x, void* y, cudaStream_t s) {
   MF_DISPATCH_N(op->n, apply_split_n, op, elem, x, y, s);
 }
+int apply_config(const mf_operator* op, int vk) { MF_DISPATCH_N(op->n, apply_config_n, op, vk); }
 mf_status launch_apply_cg(const mf_operator* op, int vk, void* p, const void* r, void* y, CgState* st, double* partials,
                           int update_p, long long* nblocks, cudaStream_t s) {
   MF_DISPATCH_N(op->n, apply_cg_n, op, vk, p, r, y, st, partials, update_p, nblocks, s);

@@ -278,14 +278,39 @@ __global__ void cg_p_kernel(const T* __restrict__ r, T* __restrict__ p, const fl
 // unit (the pencil's x, p, r, q~, and the q~ of the neighbour copies along y / z and of the
 // x-neighbours at both pencil ends) is issued before any sum, so a thread keeps up to 7n + 8
 // loads in flight.
+// With nparts > 0 the kernel first folds the apply's nparts partials of <p, A p> itself, every
+// CTA the same sum in the same order, and forms alpha = <r, z> / <p, A p> (breakdown when the
+// sum is not positive and finite; CTA 0 records it); otherwise alpha is in the state.  A separate
+// one-CTA kernel for it costs 4 us and a launch gap, a large part of an iteration of a small
+// problem.
 template <typename T, int N>
 __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
                                                const T* __restrict__ q, const float* __restrict__ dinv,
-                                               const GridInfo& g, RedScratch* sc, CgState* st, double* hist, int cta,
-                                               int ncta) {
+                                               const GridInfo& g, RedScratch* sc, CgState* st, double* hist,
+                                               const double* __restrict__ partials, int nparts, int cta, int ncta) {
   constexpr int N2 = N * N, N3 = N2 * N, K = N - 1;
+  double alpha = st->alpha, pq = 0.0;
+  if (nparts > 0) {
+    for (int i = threadIdx.x; i < nparts; i += RED_THREADS) pq += partials[i];
+  }
   if (st->flag != 0) return; // uniform: converged or stopped, nothing changes
-  const T al = scalar_from_double<T>(st->alpha);
+  if (nparts > 0) {
+    __shared__ double s_pq;
+    pq = block_sum(pq);
+    if (threadIdx.x == 0) s_pq = pq;
+    __syncthreads();
+    pq = s_pq;
+    if (!(pq > 0.0) || !isfinite(pq)) {
+      if (cta == 0 && threadIdx.x == 0) {
+        st->pq = pq;
+        st->alpha = 0.0;
+        st->flag = 2; // a CTA that starts later sees it and returns, as it would by the sum
+      }
+      return;
+    }
+    alpha = st->rz / pq;
+  }
+  const T al = scalar_from_double<T>(alpha);
   const long long tile_el = (long long)N3 * BL;                 // elements of one tile
   const long long ty_step = (long long)g.ntx * tile_el;         // one tile row along y
   const long long tz_step = (long long)g.ntx * g.nty * tile_el; // one tile layer along z
@@ -299,16 +324,15 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
   const long long dzm = lz > 0 ? (long long)K * N2 * BL - TX * TY : (long long)K * N2 * BL - tz_step + TX * TY * (TZ - 1);
   const long long dzp =
       lz < TZ - 1 ? -(long long)K * N2 * BL + TX * TY : tz_step - (long long)K * N2 * BL - TX * TY * (TZ - 1);
-  const long long units = g.ntiles * N2;
-  const long long warps = (long long)ncta * (RED_THREADS / 32);
+  // 32-bit: a unit is 32 n elements of a vector that fits the device
+  const int units = (int)(g.ntiles * N2), warps = ncta * (RED_THREADS / 32), txy = g.ntx * g.nty;
   typename AccOf<T>::type acc, accz; // <r, r> and (preconditioned) <r, z>
-  for (long long u = cta * (long long)(RED_THREADS / 32) + (threadIdx.x >> 5); u < units; u += warps) {
-    const long long t = u / N2;
-    const int jk = (int)(u - t * N2);
+  for (int u = cta * (RED_THREADS / 32) + (threadIdx.x >> 5); u < units; u += warps) {
+    const int t = u / N2;
+    const int jk = u - t * N2;
     const int j = jk % N, k = jk / N;
-    const int txy = g.ntx * g.nty;
-    const int tz = (int)(t / txy);
-    const int rm = (int)(t - (long long)tz * txy);
+    const int tz = t / txy;
+    const int rm = t - tz * txy;
     const int ty = rm / g.ntx, tx = rm - ty * g.ntx;
     const int cx = tx * TX + lx, cy = ty * TY + ly, cz = tz * TZ + lz;
     if (cx >= g.nx || cy >= g.ny || cz >= g.nz) continue; // padding lane: nothing to update
@@ -377,6 +401,10 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
     st->beta = rz / st->rz;
     st->rz = rz;
     st->rr = tot;
+    if (nparts > 0) {
+      st->pq = pq;
+      st->alpha = alpha;
+    }
     st->it += 1;
     if (hist && st->it < HIST_CAP) hist[st->it] = sqrt(tot) / st->bnorm;
     if (tot <= st->tol2) st->flag = 1;
@@ -384,13 +412,26 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
     else if (st->it >= st->maxit) st->flag = 3;
   }
 }
+// CTAs per SM of the update by registers: a lane's loads in flight grow with n.
+constexpr int update_minb(bool f32, int n) { return f32 ? (n <= 6 ? 3 : 2) : (n <= 7 ? 2 : 1); }
 template <typename T, int N>
-__global__ void __launch_bounds__(RED_THREADS) cg_update_kernel(T* __restrict__ x, T* __restrict__ r,
+__global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N)) cg_update_kernel(T* __restrict__ x, T* __restrict__ r,
                                                                 const T* __restrict__ p, const T* __restrict__ q,
                                                                 const float* __restrict__ dinv, GridInfo g,
-                                                                RedScratch* sc, CgState* st, double* hist) {
-  cg_update_body<T, N>(x, r, p, q, dinv, g, sc, st, hist, blockIdx.x, gridDim.x);
+                                                                RedScratch* sc, CgState* st, double* hist,
+                                                                const double* __restrict__ partials, int nparts) {
+  cg_update_body<T, N>(x, r, p, q, dinv, g, sc, st, hist, partials, nparts, blockIdx.x, gridDim.x);
 }
+// CTAs of an update: one warp per x-pencil unit up to one wave of resident CTAs, whose warps then
+// loop.  Several waves each
+// paid the launch and the reduction's tail (Q4 FP32 24^3, L2-resident: see cg_update_body's use).
+static int update_ctas(const mf_operator* op, int elem) {
+  const long long units = op->g.ntiles * op->n * op->n, need = (units + RED_THREADS / 32 - 1) / (RED_THREADS / 32);
+  const int wave = 152 * update_minb(elem == 4, op->n);
+  return (int)(need < 1 ? 1 : (need < wave ? need : wave));
+}
+// Partials up to which the update folds <p, A p> itself: 64 loads per thread in every CTA.
+constexpr long long UPDATE_FOLD_MAX = 16384;
 
 // alpha = <r, r> / <p, A p> from the apply's per-CTA partials of <p, A p>, folded in a fixed
 // order (breakdown when <p, A p> is not positive and finite).
@@ -443,15 +484,11 @@ __device__ __forceinline__ int find_member(const VecJob* jobs, int njobs, bool u
   }
   return lo;
 }
-__global__ void __launch_bounds__(1024) alpha_batch_kernel(const VecJob* __restrict__ jobs) {
-  const VecJob& j = jobs[blockIdx.x];
-  alpha_body(j.apart, j.apply_blocks, j.st);
-}
 template <typename T, int N>
-__global__ void __launch_bounds__(RED_THREADS) cg_update_batch_kernel(const VecJob* __restrict__ jobs, int njobs) {
+__global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N)) cg_update_batch_kernel(const VecJob* __restrict__ jobs, int njobs) {
   const VecJob& j = jobs[find_member(jobs, njobs, true)];
-  cg_update_body<T, N>((T*)j.x, (T*)j.r, (const T*)j.p, (const T*)j.q, j.dinv, j.g, j.sc, j.st, j.hist,
-                       (int)((long long)blockIdx.x - j.up0), (int)(j.up1 - j.up0));
+  cg_update_body<T, N>((T*)j.x, (T*)j.r, (const T*)j.p, (const T*)j.q, j.dinv, j.g, j.sc, j.st, j.hist, j.apart,
+                       (int)j.apply_blocks, (int)((long long)blockIdx.x - j.up0), (int)(j.up1 - j.up0));
 }
 template <typename T>
 __global__ void cg_p_batch_kernel(const VecJob* __restrict__ jobs, int njobs) {
@@ -655,26 +692,24 @@ static mf_status launch_cg_vec(const mf_operator* op, int elem, void* x, void* r
 
 template <int N>
 static mf_status cg_update_e(const mf_operator* op, int elem, void* x, void* r, void* p, void* q, const SolveWs& w,
-                             CgState* st, double* hist, cudaStream_t s) {
+                             CgState* st, double* hist, int nparts, cudaStream_t s) {
   const float* dinv = w.dinv_active;
-  // one warp per x-pencil unit, at most RED_MAX_BLOCKS CTAs (warps loop over further units)
-  long long bl = (op->g.ntiles * (long long)N * N + RED_THREADS / 32 - 1) / (RED_THREADS / 32);
-  if (bl > RED_MAX_BLOCKS) bl = RED_MAX_BLOCKS;
-  if (bl < 1) bl = 1;
+  const int bl = update_ctas(op, elem);
   if (elem == 8)
     cg_update_kernel<double, N><<<(unsigned)bl, RED_THREADS, 0, s>>>((double*)x, (double*)r, (const double*)p,
-                                                                      (const double*)q, dinv, op->g, w.sc2, st, hist);
+                                                                      (const double*)q, dinv, op->g, w.sc2, st, hist, w.apart, nparts);
   else if (elem == ELEM_DD)
     cg_update_kernel<dd, N><<<(unsigned)bl, RED_THREADS, 0, s>>>((dd*)x, (dd*)r, (const dd*)p, (const dd*)q, dinv,
-                                                                  op->g, w.sc2, st, hist);
+                                                                  op->g, w.sc2, st, hist, w.apart, nparts);
   else
     cg_update_kernel<float, N><<<(unsigned)bl, RED_THREADS, 0, s>>>((float*)x, (float*)r, (const float*)p,
-                                                                     (const float*)q, dinv, op->g, w.sc2, st, hist);
+                                                                     (const float*)q, dinv, op->g, w.sc2, st, hist,
+                                                                     w.apart, nparts);
   return cuda_check(cudaGetLastError(), "cg update launch");
 }
 static mf_status launch_cg_update(const mf_operator* op, int elem, void* x, void* r, void* p, void* q, const SolveWs& w,
-                                  CgState* st, double* hist, cudaStream_t s) {
-  MF_SWITCH_N(op->n, cg_update_e, op, elem, x, r, p, q, w, st, hist, s);
+                                  CgState* st, double* hist, int nparts, cudaStream_t s) {
+  MF_SWITCH_N(op->n, cg_update_e, op, elem, x, r, p, q, w, st, hist, nparts, s);
 }
 template <int N>
 static mf_status cg_p_e(const mf_operator* op, int elem, const void* r, void* p, const float* dinv, CgState* st,
@@ -689,13 +724,15 @@ static mf_status launch_cg_p(const mf_operator* op, int elem, const void* r, voi
                              cudaStream_t s) {
   MF_SWITCH_N(op->n, cg_p_e, op, elem, r, p, dinv, st, s);
 }
-// apply with <p, A_K p> partials, then alpha
+// apply with <p, A_K p> partials, then alpha where the update does not fold the partials itself;
+// *nparts: the partials left to the update (0: alpha is formed)
 static mf_status launch_apply_alpha(const mf_operator* op, int elem, void* p, const void* r, void* q, const SolveWs& w,
-                                   CgState* st, int fused_p, cudaStream_t s) {
+                                    CgState* st, int fused_p, int* nparts, cudaStream_t s) {
   const int vk = elem == ELEM_DD ? VK_DDS : view_of_elem(op, elem);
   long long nb = 0;
   mf_status rc = launch_apply_cg(op, vk, p, r, q, st, w.apart, fused_p, &nb, s);
-  if (rc) return rc;
+  *nparts = nb <= UPDATE_FOLD_MAX ? (int)nb : 0;
+  if (rc || *nparts) return rc;
   alpha_kernel<<<1, 1024, 0, s>>>(w.apart, nb, st);
   return cuda_check(cudaGetLastError(), "alpha launch");
 }
@@ -703,9 +740,10 @@ static mf_status launch_apply_alpha(const mf_operator* op, int elem, void* p, co
 // then p = z + beta p -- or, with fused_p, the apply forms p = r + beta p itself at load.
 static mf_status launch_cg_split(const mf_operator* op, int elem, void* x, void* r, void* p, void* q, const SolveWs& w,
                                  CgState* st, double* hist, int fused_p, cudaStream_t s) {
-  mf_status rc = launch_apply_alpha(op, elem, p, r, q, w, st, fused_p, s);
+  int nparts = 0;
+  mf_status rc = launch_apply_alpha(op, elem, p, r, q, w, st, fused_p, &nparts, s);
   if (rc) return rc;
-  if ((rc = launch_cg_update(op, elem, x, r, p, q, w, st, hist, s))) return rc;
+  if ((rc = launch_cg_update(op, elem, x, r, p, q, w, st, hist, nparts, s))) return rc;
   return fused_p ? MF_OK : launch_cg_p(op, elem, r, p, w.dinv_active, st, s);
 }
 
@@ -1030,13 +1068,6 @@ size_t batch_plan_bytes(int n, int vk) {
          a256(sizeof(VecJob) * (size_t)n);
 }
 
-static int update_blocks(const mf_operator* op) {
-  long long bl = (op->g.ntiles * (long long)op->n * op->n + RED_THREADS / 32 - 1) / (RED_THREADS / 32);
-  if (bl > RED_MAX_BLOCKS) bl = RED_MAX_BLOCKS;
-  if (bl < 1) bl = 1;
-  return (int)bl;
-}
-
 mf_status batch_plan_build(BatchPlan* plan, const BatchMember* m, int n, int elem, void* dev, void* host_stage,
                            cudaStream_t s) {
   if (n <= 0) return set_error(MF_ERR_ARG, "batch: no members");
@@ -1045,7 +1076,7 @@ mf_status batch_plan_build(BatchPlan* plan, const BatchMember* m, int n, int ele
   for (int i = 1; i < n; ++i) {
     const mf_operator* o = m[i].op;
     if (o->n != op0->n || o->path != op0->path || o->kind != op0->kind ||
-        o->variant[vk == VK_DDS ? VK_DD : vk] != op0->variant[vk == VK_DDS ? VK_DD : vk])
+        apply_config(o, vk) != apply_config(op0, vk))
       return set_error(MF_ERR_ARG, "batch: members of different classes");
   }
   BatchPlan p;
@@ -1080,7 +1111,7 @@ mf_status batch_plan_build(BatchPlan* plan, const BatchMember* m, int n, int ele
     v.n = o->n_native;
     v.apply_blocks = block0[i + 1] - block0[i];
     v.up0 = up;
-    up += update_blocks(o);
+    up += update_ctas(o, elem);
     v.up1 = up;
     v.pp0 = pp;
     pp += ew_blocks(o->n_native);
@@ -1099,7 +1130,6 @@ mf_status batch_plan_build(BatchPlan* plan, const BatchMember* m, int n, int ele
 template <int N>
 static mf_status batch_vec_n(const BatchPlan& p, cudaStream_t s) {
   const VecJob* vj = reinterpret_cast<const VecJob*>(p.dev + p.vec_off);
-  alpha_batch_kernel<<<p.n, 1024, 0, s>>>(vj);
   if (p.elem == 8) {
     cg_update_batch_kernel<double, N><<<(unsigned)p.up_blocks, RED_THREADS, 0, s>>>(vj, p.n);
     cg_p_batch_kernel<double><<<(unsigned)p.pp_blocks, 256, 0, s>>>(vj, p.n);
@@ -1329,10 +1359,11 @@ mf_status mf_cg_profile(const mf_operator* op, const void* b_dev, void* x_dev, i
     cudaEventRecord(E[0], s);
     if (e.form != MF_CG_ASSEMBLED) {
       const int fp = e.form == MF_CG_SPLIT_DUAL_FUSED;
-      st = launch_apply_alpha(op, el, e.w.p, e.w.r, e.w.q, e.w, e.w.st, fp, s);
+      int nparts = 0;
+      st = launch_apply_alpha(op, el, e.w.p, e.w.r, e.w.q, e.w, e.w.st, fp, &nparts, s);
       cudaEventRecord(E[1], s);
       cudaEventRecord(E[2], s);
-      if (st == MF_OK) st = launch_cg_update(op, el, e.x_in, e.w.r, e.w.p, e.w.q, e.w, e.w.st, nullptr, s);
+      if (st == MF_OK) st = launch_cg_update(op, el, e.x_in, e.w.r, e.w.p, e.w.q, e.w, e.w.st, nullptr, nparts, s);
       if (st == MF_OK && !fp) st = launch_cg_p(op, el, e.w.r, e.w.p, e.w.dinv_active, e.w.st, s);
     } else {
       st = launch_apply_split(op, view_of_elem(op, el), e.w.p, e.w.q, s);

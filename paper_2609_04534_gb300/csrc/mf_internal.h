@@ -216,6 +216,11 @@ mf_status launch_apply_split(const mf_operator* op, int vk, const void* x, void*
 // launched (the number of partials written)
 mf_status launch_apply_cg(const mf_operator* op, int vk, void* p, const void* r, void* y, CgState* st, double* partials,
                           int update_p, long long* nblocks, cudaStream_t s);
+// the launch configuration an apply of the view vk runs with (variant 0 resolved by degree, path
+// and size); members of one batch share it
+int apply_config(const mf_operator* op, int vk);
+template <int N>
+int apply_config_n(const mf_operator* op, int vk);
 // upper bound of the CTA count of any apply launch of op (size of CgFuse::partials)
 long long apply_max_blocks(const mf_operator* op);
 mf_status launch_dss(const mf_operator* op, int elem, void* y, cudaStream_t s);

@@ -1675,27 +1675,48 @@ static mf_status pencil_shape(const mf_operator* op, Shape<void (*)(ApplyArgs<S,
   }
   return MF_OK;
 }
-// The plane kernels, where they are built (false elsewhere)
+// Launch variant 0 in full: a plane kernel (CFG_PLANE) or the pencil configuration measured
+// fastest per degree, path and size on one GB300.  Any two give bitwise equal vectors, but a
+// batch's members must share one (their CTAs and CG partials differ): see apply_config.
+constexpr int CFG_PLANE = 6;
+// Planes need enough CTAs: one CTA's pass is a long serial stretch per thread (FP32 curved Q4:
+// 9.1 us on any mesh up to 12^3 cells, the pencil kernel 3.7; at 24^3, 216 CTAs, 13.3 against 16.4).
+// FP32: from one CTA per SM (two tiles each), always where the stretch is short (n = 2;
+// Cartesian up to n = 4).  Double-float: from 2048 tiles (Q2 Cartesian 16^3 6.4 against 4.4 us, 32^3
+// 12.0 against 12.9).
 template <typename T, int N>
 static bool use_plane(const mf_operator* op) {
-  return op->path == PATH_CARTESIAN ? UsePlane<T, N, PATH_CARTESIAN>::value
-                                    : (op->path == PATH_AFFINE ? UsePlane<T, N, PATH_AFFINE>::value
-                                                               : UsePlane<T, N, PATH_CURVED>::value);
+  const bool built = op->path == PATH_CARTESIAN ? UsePlane<T, N, PATH_CARTESIAN>::value
+                                                : (op->path == PATH_AFFINE ? UsePlane<T, N, PATH_AFFINE>::value
+                                                                           : UsePlane<T, N, PATH_CURVED>::value);
+  if (!built) return false;
+  if (std::is_same<T, dd>::value) return op->g.ntiles >= 2048;
+  return N == 2 || (op->path == PATH_CARTESIAN && N <= 4) || op->g.ntiles >= 304;
 }
-// The pencil configuration that launch variant 0 stands for where it is not a plane kernel: the
-// fastest measured on one GB300 per degree and path, for double-float (split apply, ms, the
-// configuration of Cfg 0 -> the chosen one; ~17M DoFs).  Cartesian: Q3 0.256 -> 0.181, Q4 0.311 ->
-// 0.228, Q5 0.291 -> 0.224, Q6 0.387 -> 0.315, Q7 0.379 -> 0.350, Q8 0.507 -> 0.428.  Affine: Q3
-// 0.457 -> 0.384, Q4 0.560 -> 0.468, Q6 0.766 -> 0.687, the others stay.  Curved: Q2 0.515 ->
-// 0.411, Q3 0.438 -> 0.419, Q5 0.646 -> 0.623, Q6 (Laplace) 0.771 -> 0.734, the others stay.
+// Small meshes take variant 1's smaller CTAs: FP32 below the plane kernels' line, double-float
+// up to 64 tiles (curved Q4 8^3 12.4 -> 8.4 us, Q6 19.7 -> 13.1, Cartesian Q6 11.3 -> 8.3; at 128
+// tiles curved Q4 19.9 against 21.6).  Above, double-float (split apply, ms at ~17M DoFs, base
+// configuration -> the chosen one).  Cartesian: Q3 0.256 -> 0.181, Q4 0.311 -> 0.228, Q5 0.291 ->
+// 0.224, Q6 0.387 -> 0.315, Q7 0.379 -> 0.350, Q8 0.507 -> 0.428.  Affine: Q3 0.457 -> 0.384, Q4
+// 0.560 -> 0.468, Q6 0.766 -> 0.687, the others stay.  Curved: Q2 0.515 -> 0.411, Q3 0.438 -> 0.419,
+// Q5 0.646 -> 0.623, Q6 (Laplace) 0.771 -> 0.734, the others stay.
 template <typename T, int N>
-static int variant0(const mf_operator* op) {
+static int pencil_config(const mf_operator* op) {
+  if (IsF32<T>::value) return N <= (op->path == PATH_CARTESIAN ? 7 : 6) && op->g.ntiles < 304 ? 1 : 0;
   if (!std::is_same<T, dd>::value) return 0;
+  if (op->g.ntiles <= 64) return 1;
   if (op->path == PATH_CARTESIAN) return N == 7 || N == 9 ? MF_VARIANT_OCCUPANCY : (N >= 4 ? MF_VARIANT_SMALL_CTA : 0);
   if (op->path == PATH_AFFINE) return N == 4 || N == 5 || N == 7 ? MF_VARIANT_OCCUPANCY : 0;
   if (N == 3) return MF_VARIANT_SMALL_CTA;
   if (N == 4 || N == 6) return 1;
   return N == 7 && op->kind == MF_LAPLACE ? MF_VARIANT_OCCUPANCY : 0;
+}
+// The configuration of a pencil / plane launch with this variant (the tensor-core variant's
+// operators run variant 0 where their vectors are not plain doubles).
+template <typename T, int N>
+static int config_of(const mf_operator* op, int variant) {
+  if (variant != 0 && variant != MF_VARIANT_TENSOR) return variant;
+  return use_plane<T, N>(op) ? CFG_PLANE : pencil_config<T, N>(op);
 }
 template <typename S, typename T, int N>
 static void plane_shape(const mf_operator* op, Shape<void (*)(ApplyArgs<S, T, N>)>& h) {
@@ -1752,11 +1773,6 @@ static mf_status apply_split_c(const mf_operator* op, const void* x, void* y, co
 template <typename S, typename T, int N, int V>
 static mf_status apply_split_v(const mf_operator* op, const void* x, void* y, const void* geom, const CgFuse<S>& cg,
                                long long* nblocks, cudaStream_t s) {
-  if (V == 0 && use_plane<T, N>(op)) {
-    Shape<void (*)(ApplyArgs<S, T, N>)> h;
-    plane_shape<S, T, N>(op, h);
-    return apply_launch<S, T, N>(op, h, x, y, geom, cg, nblocks, s);
-  }
   return apply_split_c<S, T, N, Cfg<T, N, V>>(op, x, y, geom, cg, nblocks, s);
 }
 
@@ -1794,7 +1810,12 @@ mf_status apply_block_n(const mf_operator* op, int vk, int cells, const void* x,
 template <typename S, typename T, int N>
 static mf_status apply_split_t(const mf_operator* op, int variant, const void* x, void* y, const void* geom,
                                const CgFuse<S>& cg, long long* nblocks, cudaStream_t s) {
-  if (variant == 0 && !use_plane<T, N>(op)) variant = variant0<T, N>(op);
+  variant = config_of<T, N>(op, variant);
+  if (variant == CFG_PLANE) {
+    Shape<void (*)(ApplyArgs<S, T, N>)> h;
+    plane_shape<S, T, N>(op, h);
+    return apply_launch<S, T, N>(op, h, x, y, geom, cg, nblocks, s);
+  }
   if (variant == 1) return apply_split_v<S, T, N, 1>(op, x, y, geom, cg, nblocks, s);
   if (variant == 2) return apply_split_v<S, T, N, 2>(op, x, y, geom, cg, nblocks, s);
   if constexpr (std::is_same<T, dd>::value) {
@@ -1802,6 +1823,13 @@ static mf_status apply_split_t(const mf_operator* op, int variant, const void* x
     if (variant == MF_VARIANT_OCCUPANCY) return apply_split_v<S, T, N, 5>(op, x, y, geom, cg, nblocks, s);
   }
   return apply_split_v<S, T, N, 0>(op, x, y, geom, cg, nblocks, s);
+}
+
+template <int N>
+int apply_config_n(const mf_operator* op, int vk) {
+  const int v = op->variant[vk == VK_DDS ? VK_DD : vk];
+  if (vk == VK_F32) return config_of<FP32C, N>(op, v);
+  return vk == VK_F64 ? config_of<double, N>(op, v) : config_of<dd, N>(op, v);
 }
 
 // vk: VK_F64 (double storage, native FP64 compute), VK_DD (double storage, double-float
@@ -1856,8 +1884,7 @@ static mf_status batch_fill_v(const BatchMember* m, int n, int vk, void* jobs_ho
     a.y = static_cast<S*>(m[i].q);
     a.geom = static_cast<const T*>(vk == VK_F32 ? op->v32.geom : op->v64.geom);
     block0_host[i] = b;
-    b += V == 0 && use_plane<T, N>(op) ? PlaneCfg<T, N>::blocks(op->g.ntiles)
-                                       : op->g.ntiles * (BL / (C::CB * C::CPL));
+    b += V == CFG_PLANE ? PlaneCfg<T, N>::blocks(op->g.ntiles) : op->g.ntiles * (BL / (C::CB * C::CPL));
   }
   block0_host[n] = b;
   return MF_OK;
@@ -1875,19 +1902,18 @@ static mf_status batch_launch_v(const mf_operator* op0, const void* jobs_dev, co
   const bool helm = op0->kind == MF_HELMHOLTZ;
   if (blocks <= 0 || njobs <= 0) return MF_OK;
   Shape<void (*)(ApplyBatch<S, T, N>)> h;
-  const bool plane = V == 0 && use_plane<T, N>(op0);
-  if (plane) {
+  if constexpr (V == CFG_PLANE) {
     using P = PlaneCfg<T, N>;
     h.threads = P::NT;
     h.smem = (op0->path == PATH_CARTESIAN ? 1 : 2) * sizeof(T) * N * N * N * P::CB;
-    if constexpr (V == 0 && UsePlane<T, N, PATH_CARTESIAN>::value)
+    if constexpr (UsePlane<T, N, PATH_CARTESIAN>::value)
       if (op0->path == PATH_CARTESIAN)
         h.kernel = helm ? apply_cartesian_plane_batch<S, T, N, true> : apply_cartesian_plane_batch<S, T, N, false>;
-    if constexpr (V == 0 && UsePlane<T, N, PATH_AFFINE>::value)
+    if constexpr (UsePlane<T, N, PATH_AFFINE>::value)
       if (op0->path == PATH_AFFINE)
         h.kernel =
             helm ? apply_general_plane_batch<S, T, N, false, true> : apply_general_plane_batch<S, T, N, false, false>;
-    if constexpr (V == 0 && UsePlane<T, N, PATH_CURVED>::value)
+    if constexpr (UsePlane<T, N, PATH_CURVED>::value)
       if (op0->path == PATH_CURVED)
         h.kernel = helm ? apply_general_plane_batch<S, T, N, true, true> : apply_general_plane_batch<S, T, N, true, false>;
   } else {
@@ -1918,7 +1944,8 @@ static mf_status batch_launch_v(const mf_operator* op0, const void* jobs_dev, co
 
 template <typename S, typename T, int N>
 static mf_status batch_fill_t(const BatchMember* m, int n, int vk, int variant, void* jobs_host, long long* block0_host) {
-  if (variant == 0 && !use_plane<T, N>(m[0].op)) variant = variant0<T, N>(m[0].op);
+  variant = config_of<T, N>(m[0].op, variant);
+  if (variant == CFG_PLANE) return batch_fill_v<S, T, N, CFG_PLANE>(m, n, vk, jobs_host, block0_host);
   if (variant == 1) return batch_fill_v<S, T, N, 1>(m, n, vk, jobs_host, block0_host);
   if (variant == 2) return batch_fill_v<S, T, N, 2>(m, n, vk, jobs_host, block0_host);
   if constexpr (std::is_same<T, dd>::value) {
@@ -1930,7 +1957,8 @@ static mf_status batch_fill_t(const BatchMember* m, int n, int vk, int variant, 
 template <typename S, typename T, int N>
 static mf_status batch_launch_t(const mf_operator* op0, int variant, const void* jobs_dev, const long long* block0_dev,
                                 int njobs, long long blocks, cudaStream_t s) {
-  if (variant == 0 && !use_plane<T, N>(op0)) variant = variant0<T, N>(op0);
+  variant = config_of<T, N>(op0, variant);
+  if (variant == CFG_PLANE) return batch_launch_v<S, T, N, CFG_PLANE>(op0, jobs_dev, block0_dev, njobs, blocks, s);
   if (variant == 1) return batch_launch_v<S, T, N, 1>(op0, jobs_dev, block0_dev, njobs, blocks, s);
   if (variant == 2) return batch_launch_v<S, T, N, 2>(op0, jobs_dev, block0_dev, njobs, blocks, s);
   if constexpr (std::is_same<T, dd>::value) {
@@ -2020,6 +2048,7 @@ mf_status layout_n(const mf_operator* op, int elem, int mode, const void* in, vo
 #define MF_INSTANTIATE_DEGREE(NN)                                                                        \
   namespace mf {                                                                                        \
   template mf_status apply_split_n<NN>(const mf_operator*, int, const void*, void*, cudaStream_t);      \
+  template int apply_config_n<NN>(const mf_operator*, int);                                              \
   template mf_status apply_block_n<NN>(const mf_operator*, int, int, const void*, void*, cudaStream_t);  \
   template mf_status apply_cg_n<NN>(const mf_operator*, int, void*, const void*, void*, CgState*, double*, \
                                     int, long long*, cudaStream_t);                                     \

@@ -314,7 +314,7 @@ int class_view(const Job* j) {
 // measured: no gain on the 100- and 400-request streams.)
 BatchClass* class_of(mf_server* sv, const Job* j) {
   const int vk = class_view(j);
-  const int variant = j->op->variant[vk == VK_DDS ? VK_DD : vk];
+  const int variant = apply_config(j->op, vk);
   for (BatchClass* c : sv->classes)
     if (c->n == j->op->n && c->path == j->op->path && c->kind == j->op->kind && c->elem == j->eng.vt &&
         c->variant == variant)
