@@ -15,6 +15,7 @@
 
 #include "mf_dd.cuh"
 #include "mf_internal.h"
+#include "mf_launch.cuh"
 #include "mf_reduce.cuh"
 #include "mf_solver.h"
 
@@ -262,6 +263,7 @@ __device__ __forceinline__ void cg_p_body(const T* __restrict__ r, T* __restrict
 template <typename T>
 __global__ void cg_p_kernel(const T* __restrict__ r, T* __restrict__ p, const float* __restrict__ dinv, long long n,
                             const CgState* st) {
+  pdl_enter();
   cg_p_body<T>(r, p, dinv, n, st, blockIdx.x, gridDim.x);
 }
 
@@ -420,6 +422,7 @@ __global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N)) c
                                                                 const float* __restrict__ dinv, GridInfo g,
                                                                 RedScratch* sc, CgState* st, double* hist,
                                                                 const double* __restrict__ partials, int nparts) {
+  pdl_enter();
   cg_update_body<T, N>(x, r, p, q, dinv, g, sc, st, hist, partials, nparts, blockIdx.x, gridDim.x);
 }
 // CTAs of an update: one warp per x-pencil unit up to one wave of resident CTAs, whose warps then
@@ -486,12 +489,14 @@ __device__ __forceinline__ int find_member(const VecJob* jobs, int njobs, bool u
 }
 template <typename T, int N>
 __global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N)) cg_update_batch_kernel(const VecJob* __restrict__ jobs, int njobs) {
+  pdl_enter();
   const VecJob& j = jobs[find_member(jobs, njobs, true)];
   cg_update_body<T, N>((T*)j.x, (T*)j.r, (const T*)j.p, (const T*)j.q, j.dinv, j.g, j.sc, j.st, j.hist, j.apart,
                        (int)j.apply_blocks, (int)((long long)blockIdx.x - j.up0), (int)(j.up1 - j.up0));
 }
 template <typename T>
 __global__ void cg_p_batch_kernel(const VecJob* __restrict__ jobs, int njobs) {
+  pdl_enter();
   const VecJob& j = jobs[find_member(jobs, njobs, false)];
   cg_p_body<T>((const T*)j.r, (T*)j.p, j.dinv, j.n, j.st, (long long)blockIdx.x - j.pp0, j.pp1 - j.pp0);
 }
@@ -695,17 +700,17 @@ static mf_status cg_update_e(const mf_operator* op, int elem, void* x, void* r, 
                              CgState* st, double* hist, int nparts, cudaStream_t s) {
   const float* dinv = w.dinv_active;
   const int bl = update_ctas(op, elem);
+  cudaError_t e;
   if (elem == 8)
-    cg_update_kernel<double, N><<<(unsigned)bl, RED_THREADS, 0, s>>>((double*)x, (double*)r, (const double*)p,
-                                                                      (const double*)q, dinv, op->g, w.sc2, st, hist, w.apart, nparts);
+    e = launch_pdl(cg_update_kernel<double, N>, bl, RED_THREADS, 0, s, (double*)x, (double*)r, (const double*)p,
+                   (const double*)q, dinv, op->g, w.sc2, st, hist, w.apart, nparts);
   else if (elem == ELEM_DD)
-    cg_update_kernel<dd, N><<<(unsigned)bl, RED_THREADS, 0, s>>>((dd*)x, (dd*)r, (const dd*)p, (const dd*)q, dinv,
-                                                                  op->g, w.sc2, st, hist, w.apart, nparts);
+    e = launch_pdl(cg_update_kernel<dd, N>, bl, RED_THREADS, 0, s, (dd*)x, (dd*)r, (const dd*)p, (const dd*)q, dinv,
+                   op->g, w.sc2, st, hist, w.apart, nparts);
   else
-    cg_update_kernel<float, N><<<(unsigned)bl, RED_THREADS, 0, s>>>((float*)x, (float*)r, (const float*)p,
-                                                                     (const float*)q, dinv, op->g, w.sc2, st, hist,
-                                                                     w.apart, nparts);
-  return cuda_check(cudaGetLastError(), "cg update launch");
+    e = launch_pdl(cg_update_kernel<float, N>, bl, RED_THREADS, 0, s, (float*)x, (float*)r, (const float*)p,
+                   (const float*)q, dinv, op->g, w.sc2, st, hist, w.apart, nparts);
+  return cuda_check(e, "cg update launch");
 }
 static mf_status launch_cg_update(const mf_operator* op, int elem, void* x, void* r, void* p, void* q, const SolveWs& w,
                                   CgState* st, double* hist, int nparts, cudaStream_t s) {
@@ -715,10 +720,11 @@ template <int N>
 static mf_status cg_p_e(const mf_operator* op, int elem, const void* r, void* p, const float* dinv, CgState* st,
                         cudaStream_t s) {
   const long long n = op->n_native;
-  if (elem == 8) cg_p_kernel<double><<<ew_blocks(n), 256, 0, s>>>((const double*)r, (double*)p, dinv, n, st);
-  else if (elem == ELEM_DD) cg_p_kernel<dd><<<ew_blocks(n), 256, 0, s>>>((const dd*)r, (dd*)p, dinv, n, st);
-  else cg_p_kernel<float><<<ew_blocks(n), 256, 0, s>>>((const float*)r, (float*)p, dinv, n, st);
-  return cuda_check(cudaGetLastError(), "cg p launch");
+  cudaError_t e;
+  if (elem == 8) e = launch_pdl(cg_p_kernel<double>, ew_blocks(n), 256, 0, s, (const double*)r, (double*)p, dinv, n, st);
+  else if (elem == ELEM_DD) e = launch_pdl(cg_p_kernel<dd>, ew_blocks(n), 256, 0, s, (const dd*)r, (dd*)p, dinv, n, st);
+  else e = launch_pdl(cg_p_kernel<float>, ew_blocks(n), 256, 0, s, (const float*)r, (float*)p, dinv, n, st);
+  return cuda_check(e, "cg p launch");
 }
 static mf_status launch_cg_p(const mf_operator* op, int elem, const void* r, void* p, const float* dinv, CgState* st,
                              cudaStream_t s) {
@@ -1130,17 +1136,19 @@ mf_status batch_plan_build(BatchPlan* plan, const BatchMember* m, int n, int ele
 template <int N>
 static mf_status batch_vec_n(const BatchPlan& p, cudaStream_t s) {
   const VecJob* vj = reinterpret_cast<const VecJob*>(p.dev + p.vec_off);
+  const unsigned up = (unsigned)p.up_blocks, pp = (unsigned)p.pp_blocks;
+  cudaError_t e, f;
   if (p.elem == 8) {
-    cg_update_batch_kernel<double, N><<<(unsigned)p.up_blocks, RED_THREADS, 0, s>>>(vj, p.n);
-    cg_p_batch_kernel<double><<<(unsigned)p.pp_blocks, 256, 0, s>>>(vj, p.n);
+    e = launch_pdl(cg_update_batch_kernel<double, N>, up, RED_THREADS, 0, s, vj, p.n);
+    f = launch_pdl(cg_p_batch_kernel<double>, pp, 256, 0, s, vj, p.n);
   } else if (p.elem == ELEM_DD) {
-    cg_update_batch_kernel<dd, N><<<(unsigned)p.up_blocks, RED_THREADS, 0, s>>>(vj, p.n);
-    cg_p_batch_kernel<dd><<<(unsigned)p.pp_blocks, 256, 0, s>>>(vj, p.n);
+    e = launch_pdl(cg_update_batch_kernel<dd, N>, up, RED_THREADS, 0, s, vj, p.n);
+    f = launch_pdl(cg_p_batch_kernel<dd>, pp, 256, 0, s, vj, p.n);
   } else {
-    cg_update_batch_kernel<float, N><<<(unsigned)p.up_blocks, RED_THREADS, 0, s>>>(vj, p.n);
-    cg_p_batch_kernel<float><<<(unsigned)p.pp_blocks, 256, 0, s>>>(vj, p.n);
+    e = launch_pdl(cg_update_batch_kernel<float, N>, up, RED_THREADS, 0, s, vj, p.n);
+    f = launch_pdl(cg_p_batch_kernel<float>, pp, 256, 0, s, vj, p.n);
   }
-  return cuda_check(cudaGetLastError(), "batched CG launch");
+  return cuda_check(e != cudaSuccess ? e : f, "batched CG launch");
 }
 
 mf_status batch_iteration(const BatchPlan& p, cudaStream_t s) {

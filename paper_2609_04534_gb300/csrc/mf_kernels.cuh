@@ -11,6 +11,7 @@
 
 #include "mf_dd.cuh"
 #include "mf_internal.h"
+#include "mf_launch.cuh"
 #include "mf_reduce.cuh"
 
 namespace mf {
@@ -856,20 +857,24 @@ __device__ __forceinline__ void cartesian_apply(const ApplyJob<S, T>& a, const T
 template <typename S, typename T, int N, int CB, int MINB, bool HELM>
 __global__ void __launch_bounds__(N * N * CB, MINB) apply_cartesian(ApplyArgs<S, T, N> A) {
   constexpr int CC = CB * CellsPer<T>::value, GPT = BL / CC; // cells per CTA, CTAs per tile
+  pdl_enter();
   cartesian_apply<S, T, N, CB, HELM>(A.j, A.tab, blockIdx.x / GPT, (blockIdx.x % GPT) * CC, blockIdx.x);
 }
 template <typename S, typename T, int N, int CB, int MINB, bool CURVED, bool HELM>
 __global__ void __launch_bounds__(N * N * CB, MINB) apply_general(ApplyArgs<S, T, N> A) {
   constexpr int CC = CB * CellsPer<T>::value, GPT = BL / CC;
+  pdl_enter();
   general_body<S, T, N, CB, CURVED, HELM>(A.j, A.tab, blockIdx.x / GPT, (blockIdx.x % GPT) * CC, blockIdx.x);
 }
 
 template <typename S, typename T, int N, bool HELM>
 __global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_C) apply_cartesian_plane(ApplyArgs<S, T, N> A) {
+  pdl_enter();
   cartesian_plane<S, T, N, HELM>(A.j, A.tab, blockIdx.x);
 }
 template <typename S, typename T, int N, bool CURVED, bool HELM>
 __global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_G) apply_general_plane(ApplyArgs<S, T, N> A) {
+  pdl_enter();
   general_plane<S, T, N, CURVED, HELM>(A.j, A.tab, blockIdx.x);
 }
 
@@ -911,6 +916,7 @@ __global__ void __launch_bounds__(N * N * CB, MINB) apply_cartesian_batch(ApplyB
   __shared__ __align__(16) ApplyJob<S, T> sj;
   __shared__ int jheld;
   if (threadIdx.x == 0) jheld = -1;
+  pdl_enter();
   for (long long u = blockIdx.x; u < B.nunits; u += gridDim.x) {
     const long long b = batch_unit(B.jobs, B.block0, B.njobs, u, sj, jheld);
     cartesian_apply<S, T, N, CB, HELM>(sj, B.tab, b / GPT, (int)(b % GPT) * CC, b);
@@ -923,6 +929,7 @@ __global__ void __launch_bounds__(N * N * CB, MINB) apply_general_batch(ApplyBat
   __shared__ __align__(16) ApplyJob<S, T> sj;
   __shared__ int jheld;
   if (threadIdx.x == 0) jheld = -1;
+  pdl_enter();
   for (long long u = blockIdx.x; u < B.nunits; u += gridDim.x) {
     const long long b = batch_unit(B.jobs, B.block0, B.njobs, u, sj, jheld);
     general_body<S, T, N, CB, CURVED, HELM>(sj, B.tab, b / GPT, (int)(b % GPT) * CC, b);
@@ -936,6 +943,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_C)
   __shared__ __align__(16) ApplyJob<S, T> sj;
   __shared__ int jheld;
   if (threadIdx.x == 0) jheld = -1;
+  pdl_enter();
   for (long long u = blockIdx.x; u < B.nunits; u += gridDim.x) {
     const long long b = batch_unit(B.jobs, B.block0, B.njobs, u, sj, jheld);
     cartesian_plane<S, T, N, HELM>(sj, B.tab, b);
@@ -948,6 +956,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, N>::NT, PlaneCfg<T, N>::MINB_G)
   __shared__ __align__(16) ApplyJob<S, T> sj;
   __shared__ int jheld;
   if (threadIdx.x == 0) jheld = -1;
+  pdl_enter();
   for (long long u = blockIdx.x; u < B.nunits; u += gridDim.x) {
     const long long b = batch_unit(B.jobs, B.block0, B.njobs, u, sj, jheld);
     general_plane<S, T, N, CURVED, HELM>(sj, B.tab, b);
@@ -1064,6 +1073,7 @@ __global__ void __launch_bounds__(DSS_THREADS) dss_kernel(T* __restrict__ y, Gri
                                                           long long nunits) {
   using D = DssCfg<N>;
   constexpr int K = N - 1, N2 = N * N, N3 = N2 * N, U = D::U, CL = D::CL, E1 = D::E > 0 ? D::E : 1;
+  pdl_enter();
   const long long u = (long long)blockIdx.x * (DSS_THREADS / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (u >= nunits) return;
@@ -1759,8 +1769,7 @@ static mf_status apply_launch(const mf_operator* op, const Shape<void (*)(ApplyA
   }
   a.j.pf_tiles = prefetch_distance_tiles((const void*)h.kernel, h.threads, h.smem, h.ctas_per_tile) * h.tiles_per_cta;
   a.j.pf_geom = (op->path == PATH_CURVED && !IsF32<T>::value) ? 1 : 0;
-  h.kernel<<<(unsigned)blocks, h.threads, h.smem, s>>>(a);
-  return cuda_check(cudaGetLastError(), "apply launch");
+  return cuda_check(launch_pdl(h.kernel, (unsigned)blocks, h.threads, h.smem, s, a), "apply launch");
 }
 template <typename S, typename T, int N, typename C>
 static mf_status apply_split_c(const mf_operator* op, const void* x, void* y, const void* geom, const CgFuse<S>& cg,
@@ -1938,8 +1947,7 @@ static mf_status batch_launch_v(const mf_operator* op0, const void* jobs_dev, co
   // one persistent launch: the CTAs resident on the GPU at once, looping over the units
   B.nunits = blocks;
   const long long grid = std::min<long long>(blocks, resident_ctas((const void*)h.kernel, h.threads, h.smem));
-  h.kernel<<<(unsigned)grid, h.threads, h.smem, s>>>(B);
-  return cuda_check(cudaGetLastError(), "batched apply launch");
+  return cuda_check(launch_pdl(h.kernel, (unsigned)grid, h.threads, h.smem, s, B), "batched apply launch");
 }
 
 template <typename S, typename T, int N>
@@ -1993,9 +2001,10 @@ static mf_status dss_mode(const mf_operator* op, int elem, void* y, int avg, cud
   const long long nlow = g.ntiles - (long long)(g.ntx - 1) * (g.nty - 1) * (g.ntz - 1);
   const long long nmain = g.ntiles * DssCfg<N>::CHUNKS, units = nmain + nlow * DssCfg<N>::LOW;
   const unsigned blocks = (unsigned)((units + DSS_THREADS / 32 - 1) / (DSS_THREADS / 32));
-  if (elem == 8) dss_kernel<double, N><<<blocks, DSS_THREADS, 0, s>>>(static_cast<double*>(y), g, avg, nmain, units);
-  else dss_kernel<float, N><<<blocks, DSS_THREADS, 0, s>>>(static_cast<float*>(y), g, avg, nmain, units);
-  return cuda_check(cudaGetLastError(), "dss launch");
+  const cudaError_t e =
+      elem == 8 ? launch_pdl(dss_kernel<double, N>, blocks, DSS_THREADS, 0, s, static_cast<double*>(y), g, avg, nmain, units)
+                : launch_pdl(dss_kernel<float, N>, blocks, DSS_THREADS, 0, s, static_cast<float*>(y), g, avg, nmain, units);
+  return cuda_check(e, "dss launch");
 }
 template <int N>
 mf_status dss_n(const mf_operator* op, int elem, void* y, cudaStream_t s) {

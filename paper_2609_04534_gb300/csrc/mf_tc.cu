@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(TC_NT, 1) apply_cartesian_tc(const __grid_cons
   using C = TcCfg<N>;
   constexpr int NN = C::NN, KP = C::KP, VPT = C::VPT, CH = C::CH;
   extern __shared__ __align__(1024) unsigned char tc_smem[];
+  pdl_enter();
   unsigned char* sA = tc_smem;                        // TC_S slices [128 cells x KP]
   unsigned char* sB = tc_smem + TC_S * C::A_SLICE;    // [T_0 | ... | T_5]: TC_S * KP rows x KP
   double* sX = reinterpret_cast<double*>(sB + TC_S * C::B_SLICE); // the group's x, native layout
@@ -496,8 +497,7 @@ mf_status tc_launch_n(const mf_operator* op, const void* x, void* y, cudaStream_
   }
   long long grid = (long long)sm_count();
   if (grid > a.ngroups) grid = a.ngroups;
-  apply_cartesian_tc<N><<<(unsigned)grid, TC_NT, C::SMEM, s>>>(a);
-  return cuda_check(cudaGetLastError(), "tensor-core apply launch");
+  return cuda_check(launch_pdl(apply_cartesian_tc<N>, (unsigned)grid, TC_NT, C::SMEM, s, a), "tensor-core apply launch");
 }
 
 } // namespace
