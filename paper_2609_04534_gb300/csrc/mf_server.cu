@@ -375,15 +375,23 @@ mf_status after_advance(mf_server* sv, Job* j, Slot& sl) {
   return cuda_check(cudaEventRecord(sl.ev, sl.s), "event record");
 }
 
-// One batched CG iteration of a class's planned composition as a CUDA graph (apply, alpha,
-// update, direction), launched chunk times per chunk.  A graph of one iteration keeps the
-// re-capture after a membership change short (a handful of launches instead of a chunk's
-// worth); an existing executable graph is updated in place when the new one differs only in
-// parameters (launch sizes), else rebuilt.
-mf_status capture_iteration(BatchClass* c) {
+// Batched CG iterations of a class's planned composition as a CUDA graph (apply, update,
+// direction, GRAPH_ITERATIONS times or the largest divisor of the chunk below it), launched
+// until the chunk is done.  A short graph keeps the re-capture after a membership change short; a
+// graph of one iteration made the scheduler thread launch ten times per chunk and class, which
+// with a handful of classes took longer than the iterations.  An existing executable graph is
+// updated in place when the new one differs only in parameters (launch sizes), else rebuilt.
+constexpr int GRAPH_ITERATIONS = 5;
+int graph_iterations(int chunk) {
+  int g = GRAPH_ITERATIONS < chunk ? GRAPH_ITERATIONS : chunk;
+  while (g > 1 && chunk % g) --g;
+  return g < 1 ? 1 : g;
+}
+mf_status capture_iteration(BatchClass* c, int iterations) {
   mf_status st = cuda_check(cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal), "batch capture");
   if (st) return st;
-  const mf_status cst = batch_iteration(c->plan, c->s);
+  mf_status cst = MF_OK;
+  for (int it = 0; it < iterations && cst == MF_OK; ++it) cst = batch_iteration(c->plan, c->s);
   cudaGraph_t g = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(c->s, &g);
   if (cst || ce != cudaSuccess) {
@@ -404,11 +412,11 @@ mf_status capture_iteration(BatchClass* c) {
   return st;
 }
 
-// A chunk: chunk launches of the iteration graph, then the members' CG states gathered and
+// A chunk: launches of the iteration graph, then the members' CG states gathered and
 // copied to the pinned mirror.
 mf_status launch_chunk(BatchClass* c, int chunk, int n) {
   mf_status st = MF_OK;
-  for (int it = 0; it < chunk && st == MF_OK; ++it) st = cuda_check(cudaGraphLaunch(c->exec, c->s), "batch launch");
+  for (int it = 0; it < chunk && st == MF_OK; it += graph_iterations(chunk)) st = cuda_check(cudaGraphLaunch(c->exec, c->s), "batch launch");
   CgState* states_dev = reinterpret_cast<CgState*>(c->dev + c->states_off);
   if (!st) st = batch_gather_states(c->plan, states_dev, c->s);
   if (!st)
@@ -471,6 +479,19 @@ bool run_batches(mf_server* sv) {
       if (pr.first == c && (int)mem.size() < c->cap) mem.push_back(pr.second);
     if (mem.empty()) continue;
     progressed = true;
+    if (mem.size() == 1) {
+      // alone in its class: its own graph chunk (the same kernels and order, so the same bits), one
+      // launch on its own stream instead of a batch's plan, launches and gather
+      Job* j = mem[0];
+      Slot& sl = sv->slots[j->slot];
+      j->batch_ready = false;
+      j->eng.external = false;
+      mf_status st = engine_advance(&j->eng);
+      j->eng.external = true;
+      if (!st) st = after_advance(sv, j, sl);
+      if (st) job_fail(sv, j, &sl, st);
+      continue;
+    }
     std::vector<uint64_t> tickets;
     for (Job* j : mem) tickets.push_back(j->ticket);
     mf_status st = MF_OK;
@@ -481,7 +502,7 @@ bool run_batches(mf_server* sv) {
       c->planned = st ? std::vector<uint64_t>() : tickets;
       c->exec_current = false;
     }
-    if (!st && !c->exec_current) st = capture_iteration(c);
+    if (!st && !c->exec_current) st = capture_iteration(c, graph_iterations(mem[0]->eng.chunk));
     if (!st) st = launch_chunk(c, mem[0]->eng.chunk, (int)mem.size());
     if (!st) st = cuda_check(cudaEventRecord(c->ev, c->s), "batch event");
     if (st) {
