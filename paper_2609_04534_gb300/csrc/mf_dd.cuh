@@ -6,8 +6,8 @@
 // (s + e = a + b exactly) and the FMA-based TwoProd (p + e = a * b exactly, e = fma(a, b, -p)).
 // fma() below accumulates a*b + c without renormalising; finish() renormalises a chain result
 // with Dekker's FastTwoSum.  Conversions to and from double split the IEEE bit pattern with
-// integer operations, so the hot loop issues no FP64 instruction except one add per stored
-// value.
+// integer operations (on the way in) or by the otherwise idle FP64 pipe (on the way out), so the
+// hot loop issues no FP64 instruction.
 #pragma once
 #include <cstring>
 
@@ -59,6 +59,26 @@ __device__ __forceinline__ dd fma(dd a, dd b, dd c) {
   return dd(s, t + (c.lo + e));
 }
 
+// The same in 10 instructions instead of 12, for chains of up to three terms: TwoSum's last
+// difference p - v and TwoProd's error a.hi b.hi - p are taken together, as a.hi b.hi - v in one
+// fma, and the cross terms go straight into lo.  lo is rounded once more per term, which shows in long
+// chains (relative error of the Cartesian apply against 64 bits, n = 7, 8: 1.06-1.11 times that of
+// fma(); n <= 5: 0.94-1.04), so it is used by kernels of n <= 5 and by the forward sweeps of the
+// Cartesian kernel at n = 6..8, where the rounded conversion of the input outweighs it (split apply,
+// FP64: Q4 curved 52^3 0.537 -> 0.509 ms, Q4 Cartesian 52^3 0.226 -> 0.212, Q2 curved 88^3 0.409 -> 0.387).
+__device__ __forceinline__ dd fma_short(dd a, dd b, dd c) {
+  const float p = a.hi * b.hi;
+  const float s = __fadd_rn(c.hi, p);
+  const float v = s - c.hi;
+  const float t = (c.hi - (s - v)) + fmaf(a.hi, b.hi, -v);
+  return dd(s, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, c.lo)) + t);
+}
+// fma() or, for double-float with SHORT, fma_short()
+template <bool SHORT>
+__device__ __forceinline__ dd fma_n(dd a, dd b, dd c) { return SHORT ? fma_short(a, b, c) : fma(a, b, c); }
+template <bool SHORT, typename A, typename B>
+__device__ __forceinline__ B fma_n(A a, B b, B c) { return fma(a, b, c); }
+
 // a*b as the first term of a chain: TwoProd of the leading parts plus the cross terms, not
 // renormalised (an fma() into a zero accumulator would spend a TwoSum on the zero).
 __device__ __forceinline__ dd mul0(dd a, dd b) {
@@ -96,8 +116,9 @@ __device__ __forceinline__ dd operator+(dd a, dd b) {
 }
 
 // double -> dd: hi keeps the leading 24 significant bits (truncated), lo the remaining 29
-// bits rounded to 24.  Magnitudes below 2^-126 flush to zero; inf/nan go through hi.
-__device__ __forceinline__ dd dd_from_double(double x) {
+// bits rounded to 24.  Magnitudes below 2^-126 flush to zero; inf/nan go through hi.  The
+// general form; dd_from_double takes the common range without its branches.
+__device__ __forceinline__ dd dd_from_double_any(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned hi32 = (unsigned)(b >> 32), lo32 = (unsigned)b;
   const int e = (int)((hi32 >> 20) & 0x7ffu);
@@ -114,6 +135,31 @@ __device__ __forceinline__ dd dd_from_double(double x) {
   return dd(h, sign ? -l : l);
 }
 
+static __device__ __noinline__ dd dd_from_double_call(double x) { return dd_from_double_any(x); }
+// Biased exponents 949..1149 (magnitudes 2^-74..2^127, where hi and lo are normal floats) without
+// the branches: hi is the double's leading 24 bits shifted left by 3 with the exponent rebased by
+// one exclusive or, lo the remaining bits as an integer times the double's power of two, 2^-52 of
+// it.  NEAR: hi is rounded instead of truncated (half its last place added first; the rounding
+// may carry, so lo keeps the double's own power), which halves the remainder and its rounding:
+// the apply's error against 64 bits falls by 4-7% at n >= 4 (no change below, where it is not used).
+// INL: the general form in line or called.
+template <bool INL = false, bool NEAR = false>
+__device__ __forceinline__ dd dd_from_double(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x), n = NEAR ? b + (1ull << 28) : b;
+  const unsigned hi32 = (unsigned)(b >> 32), nh = (unsigned)(n >> 32);
+  const unsigned h = ((__funnelshift_l((unsigned)n, nh, 3) ^ 0x40000000u) & 0x7fffffffu) | (nh & 0x80000000u);
+  dd r(__uint_as_float(h), 0.0f);
+  if (NEAR) {
+    const float l = __int2float_rn((int)((unsigned)b << 3) >> 3) *
+                    __uint_as_float((((hi32 << 3) ^ 0x40000000u) & 0x7f800000u) - (52u << 23));
+    r.lo = __uint_as_float(__float_as_uint(l) ^ (hi32 & 0x80000000u));
+  } else {
+    r.lo = __uint2float_rn((unsigned)b & 0x1fffffffu) * __uint_as_float((h & 0xff800000u) - (52u << 23));
+  }
+  if ((hi32 & 0x7fffffffu) - (949u << 20) >= (201u << 20)) r = INL ? dd_from_double_any(x) : dd_from_double_call(x);
+  return r;
+}
+
 // float -> double by bit manipulation (normal numbers; zero and subnormals give zero).
 __host__ __device__ __forceinline__ double f2d_bits(float f) {
   const unsigned u = fbits(f);
@@ -127,10 +173,21 @@ __host__ __device__ __forceinline__ double f2d_bits(float f) {
 }
 
 // dd -> double: exact sum of the two parts (one FP64 add, rounded to nearest).  A subnormal lo
-// flushes to zero, as in dd_from_double.  (An integer-only form of this conversion, lo added
-// as a count of ulps of hi's double, was measured: 20 integer instructions cost the
-// issue-bound apply kernels more than the FP64 add, 3-6%.)
-__host__ __device__ __forceinline__ double dd_to_double(dd a) { return f2d_bits(a.hi) + f2d_bits(a.lo); }
+// flushes to zero, as in dd_from_double.  On the device the parts are converted by the FP64
+// pipe, which the apply otherwise leaves idle (3 of its slow instructions per stored value take 1.5 clocks
+// of an SM, an apply 2.5 or more per value); the same conversion by bits takes about 20
+// instructions of the issue-bound kernels (split apply, FP64: Q4 Cartesian 52^3 0.205 -> 0.193 ms, Q2
+// 88^3 0.160 -> 0.137, Q2 sheared 88^3 0.329 -> 0.307).
+__host__ __device__ __forceinline__ double dd_to_double(dd a) {
+#ifdef __CUDA_ARCH__
+  double h, l;
+  asm("cvt.ftz.f64.f32 %0, %1;" : "=d"(h) : "f"(a.hi));
+  asm("cvt.ftz.f64.f32 %0, %1;" : "=d"(l) : "f"(a.lo));
+  return h + l;
+#else
+  return f2d_bits(a.hi) + f2d_bits(a.lo);
+#endif
+}
 
 // Two FP32 values of neighbouring cells processed by one thread (the FP32 apply): every
 // operation acts on both lanes; table coefficients stay scalar floats.  Products and sums that

@@ -134,11 +134,11 @@ __device__ __forceinline__ float add_lazy(float a, float b) { return a + b; }
 __device__ __forceinline__ float sub_lazy(float a, float b) { return a - b; }
 
 // sum_i c[i] x[i], i < M (M >= 1), not renormalised
-template <typename C, typename T, int M>
+template <typename C, typename T, bool SHORT, int M>
 __device__ __forceinline__ T chain(const C* c, const T* x) {
   T s = mul0(c[0], x[0]);
 #pragma unroll
-  for (int i = 1; i < M; ++i) s = fma(c[i], x[i], s);
+  for (int i = 1; i < M; ++i) s = fma_n<SHORT>(c[i], x[i], s);
   return s;
 }
 __device__ __forceinline__ f2 add_lazy(f2 a, f2 b) { return a + b; }
@@ -163,14 +163,28 @@ struct Fold {
   __device__ __forceinline__ void apply(const EoTab<C, N>& t, T* out) const {
 #pragma unroll
     for (int q = 0; q < H; ++q) {
-      const T u = chain<C, T, HE>(t.F + q * HE, e);
-      const T w = chain<C, T, H>(t.G + q * H, o);
+      const T u = chain<C, T, (N <= 5), HE>(t.F + q * HE, e);
+      const T w = chain<C, T, (N <= 5), H>(t.G + q * H, o);
       out[q] = finish(add_lazy(u, w));
       out[N - 1 - q] = finish(ANTI ? sub_lazy(w, u) : sub_lazy(u, w));
     }
-    if (N % 2) out[H] = finish(ANTI ? chain<C, T, H>(t.Mid, o) : chain<C, T, HE>(t.Mid, e));
+    if (N % 2) out[H] = finish(ANTI ? chain<C, T, (N <= 5), H>(t.Mid, o) : chain<C, T, (N <= 5), HE>(t.Mid, e));
   }
 };
+
+// Whether a kernel carries dd_from_double's general form in line (its registers) or calls it
+// (its code).  Split apply, FP64, ms in line / called: Cartesian Q3 64^3 0.153 / 0.162, Q4 52^3 0.193 /
+// 0.198, Q7 33^3 0.297 / 0.286, Q8 30^3 0.374 / 0.345; curved Q1 120^3 0.251 / 0.221, Q3 64^3 0.387 /
+// 0.370.
+template <int N>
+struct InlineFrom { static constexpr bool cartesian = N <= 7; };
+template <bool INL, bool NEAR, typename T, typename S>
+__device__ __forceinline__ T load_value(S v) {
+  if constexpr (std::is_same<T, dd>::value && std::is_same<S, double>::value)
+    return dd_from_double<INL, NEAR>(v);
+  else
+    return to_compute<T, S>(v);
+}
 
 // Load the CB values (CB * CPL cells from lane0) of tile t into smem as buf[l*CB + c] (cell
 // fastest; a pair value holds cells lane0 + 2c and lane0 + 2c + 1), zeroing padding cells and,
@@ -178,7 +192,7 @@ struct Fold {
 // vector is the new direction p = r + beta p, written back.
 // Thread (l0, c) = (threadIdx.x / CB, threadIdx.x % CB) loads local dofs l0 + m n^2 of value c
 // (m < n): its cell is the same in every trip, so its coordinates are found once.
-template <typename S, typename T, int N, int CB, int NT>
+template <bool INL, typename S, typename T, int N, int CB, int NT>
 __device__ __forceinline__ void load_tile(const ApplyJob<S, T>& a, long long t, int lane0, T* buf) {
   constexpr int N2 = N * N, N3 = N2 * N, CPL = CellsPer<T>::value;
   static_assert(NT == N2 * CB, "one thread per pencil position and value");
@@ -204,7 +218,7 @@ __device__ __forceinline__ void load_tile(const ApplyJob<S, T>& a, long long t, 
         } else {
           xv = a.x[e];
         }
-        v = to_compute<T, S>(xv);
+        v = load_value<INL, (N >= 4), T, S>(xv);
         if (a.g.bc) {
           const int i = l % N, j = (l / N) % N, k = l / N2;
           if (on_cube_boundary<N>(a.g, cx, cy, cz, i, j, k)) v = T(0);
@@ -265,7 +279,7 @@ __device__ __forceinline__ void load_xpencil(const ApplyJob<S, T>& a, long long 
         } else {
           xv = a.x[e];
         }
-        v = to_compute<T, S>(xv);
+        v = load_value<InlineFrom<N>::cartesian, (N >= 4), T, S>(xv);
         if (a.g.bc && on_cube_boundary<N>(a.g, cx, cy, cz, i, j, k)) v = T(0);
       } else if (fuse) {
         pg[e] = S(0);
@@ -376,7 +390,7 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
   T* buf1 = buf0 + N3 * CB;
   if (a.cg.st != nullptr && a.cg.st->flag != 0) return; // CG step after convergence: no work
   prefetch_next_wave<S, T, N, 0>(a, t, lane0);
-  load_tile<S, T, N, CB, NT>(a, t, lane0, buf0);
+  load_tile<InlineFrom<N>::cartesian, S, T, N, CB, NT>(a, t, lane0, buf0);
   __syncthreads();
   const int c = threadIdx.x % CB, p = threadIdx.x / CB, pa = p % N, pb = p / N;
   { // x: pencil (j=pa, k=pb): M and K share one fold of the pencil
@@ -468,9 +482,9 @@ __device__ __forceinline__ void fd_forward(const FdTab<C, N>& t, const T* in, T*
   constexpr int H = N / 2, HE = (N + 1) / 2;
   const Fold<T, N, false> f(in);
 #pragma unroll
-  for (int m = 0; m < HE; ++m) out[m] = finish(chain<C, T, HE>(t.Ff + m * HE, f.e));
+  for (int m = 0; m < HE; ++m) out[m] = finish(chain<C, T, (N <= 8), HE>(t.Ff + m * HE, f.e));
 #pragma unroll
-  for (int m = 0; m < H; ++m) out[HE + m] = finish(chain<C, T, H>(t.Gf + m * H, f.o));
+  for (int m = 0; m < H; ++m) out[HE + m] = finish(chain<C, T, (N <= 8), H>(t.Gf + m * H, f.o));
 }
 // backward: nodal values of a pencil from its modes
 template <typename C, typename T, int N>
@@ -478,12 +492,12 @@ __device__ __forceinline__ void fd_backward(const FdTab<C, N>& t, const T* z, T*
   constexpr int H = N / 2, HE = (N + 1) / 2;
 #pragma unroll
   for (int j = 0; j < H; ++j) {
-    const T u = chain<C, T, HE>(t.Fb + j * HE, z);
-    const T v = chain<C, T, H>(t.Gb + j * H, z + HE);
+    const T u = chain<C, T, (N <= 5), HE>(t.Fb + j * HE, z);
+    const T v = chain<C, T, (N <= 5), H>(t.Gb + j * H, z + HE);
     out[j] = finish(add_lazy(u, v));
     out[N - 1 - j] = finish(sub_lazy(u, v));
   }
-  if (N % 2) out[H] = finish(chain<C, T, HE>(t.Fb + H * HE, z));
+  if (N % 2) out[H] = finish(chain<C, T, (N <= 5), HE>(t.Fb + H * HE, z));
 }
 
 template <typename S, typename T, int N, int CB, bool HELM>
@@ -503,7 +517,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
   // slower (its registers cost resident CTAs); the FP32 view was not measured.
   constexpr bool direct = N >= 6 && N <= 8 && !IsF32<T>::value;
   if constexpr (!direct) {
-    load_tile<S, T, N, CB, NT>(a, t, lane0, buf0);
+    load_tile<InlineFrom<N>::cartesian, S, T, N, CB, NT>(a, t, lane0, buf0);
     __syncthreads();
   }
   { // forward x: pencil (j=pa, k=pb)
@@ -660,7 +674,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
   if (a.cg.st != nullptr && a.cg.st->flag != 0) return; // CG step after convergence: no work
   // streamed geometry exists only for the FP64 views (the FP32 view computes its metric)
   prefetch_next_wave<S, T, N, (CURVED && !IsF32<T>::value) ? NC : 0>(a, t, lane0);
-  load_tile<S, T, N, CB, NT>(a, t, lane0, buf0);
+  load_tile<false, S, T, N, CB, NT>(a, t, lane0, buf0);
   __syncthreads();
   const int c = threadIdx.x % CB, p = threadIdx.x / CB, pa = p % N, pb = p / N;
   { // x-sweep with S, pencil (j=pa, k=pb), in place
@@ -764,9 +778,9 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
         g3 = w * a.G[3]; g4 = w * a.G[4]; g5 = w * a.G[5];
         if (HELM) m = w * a.mdet;
       }
-      v1 = finish(fma(g0, d1, fma(g1, d2, mul0(g2, d3q))));
-      v2 = finish(fma(g1, d1, fma(g3, d2, mul0(g4, d3q))));
-      v3 = finish(fma(g2, d1, fma(g4, d2, mul0(g5, d3q))));
+      v1 = finish(fma_n<(N <= 5)>(g0, d1, fma_n<(N <= 5)>(g1, d2, mul0(g2, d3q))));
+      v2 = finish(fma_n<(N <= 5)>(g1, d1, fma_n<(N <= 5)>(g3, d2, mul0(g4, d3q))));
+      v3 = finish(fma_n<(N <= 5)>(g2, d1, fma_n<(N <= 5)>(g4, d2, mul0(g5, d3q))));
     }
     buf0[l * CB + c] = v1;
     buf2[l * CB + c] = v2;
@@ -1707,17 +1721,17 @@ static bool use_plane(const mf_operator* op) {
 // up to 64 tiles (curved Q4 8^3 12.4 -> 8.4 us, Q6 19.7 -> 13.1, Cartesian Q6 11.3 -> 8.3; at 128
 // tiles curved Q4 19.9 against 21.6).  Above, double-float (split apply, ms at ~17M DoFs, base
 // configuration -> the chosen one).  Cartesian: Q3 0.256 -> 0.181, Q4 0.311 -> 0.228, Q5 0.291 ->
-// 0.224, Q6 0.387 -> 0.315, Q7 0.379 -> 0.350, Q8 0.507 -> 0.428.  Affine: Q3 0.457 -> 0.384, Q4
+// 0.224, Q6 0.387 -> 0.315, Q7 0.379 -> 0.350, Q8 0.507 -> 0.428.  Affine: Q3 0.392 -> 0.348, Q4
 // 0.560 -> 0.468, Q6 0.766 -> 0.687, the others stay.  Curved: Q2 0.515 -> 0.411, Q3 0.438 -> 0.419,
-// Q5 0.646 -> 0.623, Q6 (Laplace) 0.771 -> 0.734, the others stay.
+// Q4 (Laplace) 0.513 -> 0.483, Q5 0.646 -> 0.623, Q6 (Laplace) 0.771 -> 0.734, the others stay.
 template <typename T, int N>
 static int pencil_config(const mf_operator* op) {
   if (IsF32<T>::value) return N <= (op->path == PATH_CARTESIAN ? 7 : 6) && op->g.ntiles < 304 ? 1 : 0;
   if (!std::is_same<T, dd>::value) return 0;
   if (op->g.ntiles <= 64) return 1;
   if (op->path == PATH_CARTESIAN) return N == 7 || N == 9 ? MF_VARIANT_OCCUPANCY : (N >= 4 ? MF_VARIANT_SMALL_CTA : 0);
-  if (op->path == PATH_AFFINE) return N == 4 || N == 5 || N == 7 ? MF_VARIANT_OCCUPANCY : 0;
-  if (N == 3) return MF_VARIANT_SMALL_CTA;
+  if (op->path == PATH_AFFINE) return N == 4 ? MF_VARIANT_SMALL_CTA : (N == 5 || N == 7 ? MF_VARIANT_OCCUPANCY : 0);
+  if (N == 3 || (N == 5 && op->kind == MF_LAPLACE)) return MF_VARIANT_SMALL_CTA;
   if (N == 4 || N == 6) return 1;
   return N == 7 && op->kind == MF_LAPLACE ? MF_VARIANT_OCCUPANCY : 0;
 }

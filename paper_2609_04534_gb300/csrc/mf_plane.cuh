@@ -81,7 +81,7 @@ struct PlaneMask {
 
 // The plane k of a value into u[j][i]: load_tile's values (padding cells and constrained nodes
 // zero; in a CG step with update_p the new direction p = r + beta p, written back).
-template <typename S, typename T, int N>
+template <bool INL, typename S, typename T, int N>
 __device__ __forceinline__ void load_plane(const ApplyJob<S, T>& a, const PlaneCell& q, int k, T (&u)[N][N]) {
   constexpr int N2 = N * N, N3 = N2 * N, CPL = CellsPer<T>::value;
   const bool fuse = a.cg.st != nullptr && a.cg.update_p;
@@ -115,7 +115,7 @@ __device__ __forceinline__ void load_plane(const ApplyJob<S, T>& a, const PlaneC
 #pragma unroll
     for (int j = 0; j < N; ++j)
 #pragma unroll
-      for (int i = 0; i < N; ++i) u[j][i] = to_compute<T, S>(x[j][i]);
+      for (int i = 0; i < N; ++i) u[j][i] = load_value<INL, (N >= 4), T, S>(x[j][i]);
     if (m.on) {
 #pragma unroll
       for (int j = 0; j < N; ++j)
@@ -262,7 +262,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
   B += c;
   {
     T u[N][N];
-    load_plane<S, T, N>(a, cell, p, u);
+    load_plane<false, S, T, N>(a, cell, p, u);
     plane_x<false>(tab.eS, u);
     plane_y<false>(tab.eS, u);
 #pragma unroll
@@ -349,9 +349,9 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
             g3 = w * a.G[3]; g4 = w * a.G[4]; g5 = w * a.G[5];
             if (HELM) m = w * a.mdet;
           }
-          v1 = finish(fma(g0, e1, fma(g1, e2, mul0(g2, e3))));
-          v2 = finish(fma(g1, e1, fma(g3, e2, mul0(g4, e3))));
-          v3 = finish(fma(g2, e1, fma(g4, e2, mul0(g5, e3))));
+          v1 = finish(fma_n<(N <= 5)>(g0, e1, fma_n<(N <= 5)>(g1, e2, mul0(g2, e3))));
+          v2 = finish(fma_n<(N <= 5)>(g1, e1, fma_n<(N <= 5)>(g3, e2, mul0(g4, e3))));
+          v3 = finish(fma_n<(N <= 5)>(g2, e1, fma_n<(N <= 5)>(g4, e2, mul0(g5, e3))));
         }
         d1[i] = v1;
         d2[j][i] = v2;
@@ -423,7 +423,7 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
   A += c;
   {
     T u[N][N];
-    load_plane<S, T, N>(a, cell, p, u);
+    load_plane<InlineFrom<N>::cartesian, S, T, N>(a, cell, p, u);
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       T out[N];
