@@ -131,7 +131,9 @@ __device__ __forceinline__ dd dd_from_double_any(double x) {
   const float h = __uint_as_float(sign | ((unsigned)ef << 23) | mant);
   const unsigned r = lo32 & 0x1fffffffu;
   const int es = e - 948; // float biased exponent of 2^(e - 1075)
-  float l = (es > 0) ? __uint2float_rn(r) * __uint_as_float((unsigned)es << 23) : 0.0f;
+  // below 2^-74 lo's power of two is no normal float: scaled in two steps (lo itself may be subnormal)
+  float l = (es > 0) ? __uint2float_rn(r) * __uint_as_float((unsigned)es << 23)
+            : (es > -64) ? __uint2float_rn(r) * 0x1p-64f * __uint_as_float((unsigned)(es + 64) << 23) : 0.0f;
   return dd(h, sign ? -l : l);
 }
 

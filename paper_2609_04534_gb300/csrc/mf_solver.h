@@ -59,6 +59,7 @@ struct SolverEngine {
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
   bool record = false, cancel = false;
+  bool direct = false;   // chunks as direct launches (mf_cg_solve) instead of one graph (the server)
   bool external = false; // inner CG iterations are run by a batch (the server), not by chunks
   bool idle = false;     // the last advance enqueued nothing (external inner CG waiting for a batch)
   int hist_off = 0;
