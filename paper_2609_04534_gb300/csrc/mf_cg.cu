@@ -872,16 +872,19 @@ static mf_status eng_iteration(SolverEngine* e, cudaStream_t s) {
   return launch_cg_vec(e->op, e->elem_in, e->x_in, e->w.r, e->w.p, e->w.q, e->w.sc1, e->w.sc2, e->w.st, e->w.hist, s);
 }
 
-// A chunk of iterations, then the CG state to the host mirror.  mf_cg_solve launches the kernels
-// directly (e->direct): three launches take the host less time than an iteration takes the GPU even on
-// the smallest mesh, each starts while its predecessor drains (mf_launch.cuh), nothing is captured
-// and instantiated per solve (about 0.3 ms), and the last chunk stops at maxit.  The server, one
-// thread for many requests, launches a chunk as one graph.  Q2 8^3, 50 iterations: 1.15 -> 0.67 ms.
+// A chunk of iterations, then the CG state to the host mirror: as one graph launch or, for the first
+// chunks of mf_cg_solve (e->direct of them) and a short rest, as direct launches, which stop at
+// maxit.  Capturing and instantiating the graph costs about 0.3 ms per solve, a third of 50
+// iterations on an 8^3 mesh; against that the host needs 17-23 us for the three launches of an
+// iteration, which on such a mesh takes the GPU 15 us from a graph (with the kernels' early start,
+// mf_launch.cuh; 24 us without).  Q2 8^3, 50 iterations: 1.15 -> 0.96 ms.  The server, one thread for many
+// requests, always uses the graph.
 static mf_status eng_chunk(SolverEngine* e) {
   cudaStream_t s = e->s;
   mf_status st;
-  if (e->direct) {
-    const int left = e->hm->st.maxit - e->hm->st.it;
+  const int left = e->hm->st.maxit - e->hm->st.it;
+  if (e->direct > 0 && !e->exec && (e->direct > 1 || left <= 3 * e->chunk)) {
+    if (e->direct > 1) --e->direct;
     const int n = e->chunk < left ? e->chunk : (left > 1 ? left : 1);
     for (int c = 0; c < n; ++c)
       if ((st = eng_iteration(e, s))) return st;
@@ -1321,7 +1324,7 @@ mf_status mf_cg_solve_ex(const mf_operator* op, const void* b_dev, void* x_dev, 
     e.precond = opts->precond;
     e.reliable = opts->mixed_restart == 0;
   }
-  e.direct = true;
+  e.direct = 3; // two chunks
   e.record = g_hist_host != nullptr;
   mf_status st = engine_start(&e);
   // every advance either finishes or moves the iteration count forward by a chunk; bound the

@@ -59,7 +59,7 @@ struct SolverEngine {
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
   bool record = false, cancel = false;
-  bool direct = false;   // chunks as direct launches (mf_cg_solve) instead of one graph (the server)
+  int direct = 0; // 0: chunks are graph launches; d > 0: d - 1 chunks, and a short rest, are direct ones
   bool external = false; // inner CG iterations are run by a batch (the server), not by chunks
   bool idle = false;     // the last advance enqueued nothing (external inner CG waiting for a batch)
   int hist_off = 0;
