@@ -900,10 +900,12 @@ def main():
             "serve_burst_unbatched": serve_unbatched,
             "cpu_baseline": cpu,
             "e2e": e2e,
-            # mask, max|b|, zero x, scale b, copy p, <r,r>, state; then 4 kernels per iteration
-            # (apply, alpha, update, p) in graph chunks of 20 iterations (a partial last chunk
-            # still launches its kernels); the final conversion of x
-            "gpu_launches": 7 + 4 * 20 * ((its + 19) // 20) + 1,
+            # mask, max|b|, zero x, scale b, copy p, <r,r>, state; then per iteration apply, update and
+            # direction, and alpha where the apply leaves more than 16384 partials (8 cells per CTA:
+            # every launch variant here but 5); two chunks of 20 iterations and a rest of up to 60 are
+            # launched as they are, others by whole chunks; the final conversion of x
+            "gpu_launches": 7 + (3 if variant == mf.MF_VARIANT_OCCUPANCY else 4) *
+            (its if its <= 100 else 40 + 20 * ((its - 40 + 19) // 20)) + 1,
             "clocks": clk.summary(),
             "peaks": pk,
         }

@@ -325,11 +325,12 @@ mf_status mf_cg_solve_host(const mf_operator* op, const void* b_host, void* x_ho
  *     A p split (no duplicate summation) and forms <p, A p> -- the pairing of the consistent p
  *     with the split product over all copies (Lemma 1) -- as the sum over quadrature points
  *     of grad u . G grad u; the duplicate summation is folded into the update of x and r;
- *     then p = r + beta p.  Four kernels per iteration (apply, alpha, update, direction).
+ *     then p = r + beta p.  Three kernels per iteration (apply, update, direction), and a fourth
+ *     for alpha where the apply leaves more than 16384 partial sums of <p, A p>.
  *   MF_CG_ASSEMBLED -- apply, duplicate summation, then the vector kernels on assembled
  *     vectors (five kernels per iteration).
  *   MF_CG_SPLIT_DUAL_FUSED -- MF_CG_SPLIT_DUAL with p = r + beta p formed by the apply at
- *     load (three kernels per iteration).
+ *     load (one kernel fewer).
  * All compute the same iterates up to rounding (only <p, A p> is summed differently). */
 enum { MF_CG_DEFAULT = 0, MF_CG_SPLIT_DUAL = 1, MF_CG_ASSEMBLED = 2, MF_CG_SPLIT_DUAL_FUSED = 3 };
 /* Preconditioner (mf_solve_options.precond): none (default), Jacobi -- z = r / diag(P A P)
@@ -362,7 +363,7 @@ mf_status mf_cg_solve_ex(const mf_operator* op, const void* b_dev, void* x_dev, 
  * runs `iterations` FP64 (FP32 for an MF_FP32 operator) CG iterations from x = 0 on b, of the
  * form cg_form (MF_CG_*), launching every kernel directly (no graph) with CUDA events around
  * each kernel group on `stream`, and writes the mean durations in milliseconds:
- * ms_out[0] the apply kernel (split-dual forms: the apply and the one-CTA alpha kernel after it),
+ * ms_out[0] the apply kernel (split-dual forms: with the one-CTA alpha kernel where there is one),
  * ms_out[1] the duplicate
  * summation (assembled form; 0 for split-dual), ms_out[2] the vector kernels, ms_out[3] the
  * whole iteration.  1 <= iterations <= 1000.  Same workspace as mf_cg_solve (mixed = 0).
@@ -380,8 +381,8 @@ mf_status mf_cg_record_history(double* hist_host, int cap);
  * request keeps its geometry, vectors and CG state resident in its arena block.  Its set-up,
  * the outer steps of defect correction and its finish run on its slot's CUDA stream; its CG
  * iterations run in a continuous batch: every active request of the same degree, path,
- * operator kind, vector precision and launch variant takes part in one batched launch per
- * kernel of the (split-dual) CG iteration -- apply, alpha, update, direction -- in chunks of
+ * operator kind, vector precision and launch configuration takes part in one batched launch per
+ * kernel of the (split-dual) CG iteration -- apply, update, direction -- in chunks of
  * chunk_iterations, and requests join and leave the batch between chunks.  The batched apply
  * is one persistent launch: the CTAs that fit the GPU at once loop over the CTA-sized work
  * units of all members.  Requests whose own apply takes more than 1024 CTAs run their own

@@ -25,7 +25,7 @@ namespace mf {
 // kernel: see variant0 and mf_plane.cuh); variant 1 = CB0/2 cells per CTA, capped for 3 resident CTAs per SM;
 // variant 2 = CB0/2 cells per CTA with no register cap (high degrees spill under a cap);
 // variant 4 (double-float compute only) = CB0/2 cells per CTA, registers capped for 1.5x
-// variant 0's resident threads per SM; variant 5 (double-float only) = CB0 cells per CTA,
+// Cfg 0's resident threads per SM; variant 5 (double-float only) = CB0 cells per CTA,
 // capped for three resident CTAs (also 1.5x).  The block-size sweep of Sec. 6 found the
 // double-float apply faster in smaller blocks, and a later sweep of the register budget
 // found it faster at higher occupancy: the Cartesian apply at k = 4..7 gains 5-17%.
@@ -1650,8 +1650,8 @@ static void fill_tab(const mf_operator* op, Tab<T, N>& tab) {
 }
 
 // Block-size sweep of Sec. 6 (B cells per CTA; a measurement entry): the registers are capped
-// so that the resident threads per SM equal those of launch variant 0 (MINB * NT = 2 * NT of
-// variant 0), which separates the block size from the register budget.
+// so that the resident threads per SM equal those of the base configuration (MINB * NT = 2 * NT of
+// Cfg 0), which separates the block size from the register budget.
 template <typename T, int N, int B, bool G>
 struct BCfg {
   static constexpr int CPL = CellsPer<T>::value;

@@ -7,7 +7,7 @@
 // in its own arena block and runs the solver engine (FP64 CG, or FP32 CG inside FP64
 // defect correction).  Its set-up, outer defect-correction steps and finish run on its
 // slot's stream.  Its CG iterations run in a continuous batch: the requests in the inner-CG
-// phase are grouped by class (degree, path, kind, vector type, launch variant), and each
+// phase are grouped by class (degree, path, kind, vector type, launch configuration), and each
 // class runs chunks of batched iterations -- one launch per kernel for all its members --
 // on the class's stream; requests join and leave between chunks.  A scheduler thread
 // (native) polls one event per slot and per class, advances requests when their scalars
@@ -238,8 +238,7 @@ mf_status job_start(mf_server* sv, Job* j, Slot& sl, HostMirror* hm) {
   // CTAs at most: those are launch- and latency-bound alone, and batched with others they
   // share launches.  A larger request fills the GPU by itself and runs its own graph chunks
   // (batched with small ones it would hold them to its own chunk time).
-  // (the default launch variant puts 8 to 32 cells of a 32-cell tile in one CTA: at most 4
-  // CTAs per tile below degree 8)
+  // (a nominal count: launch configurations put 4 to 64 cells in one CTA)
   const long long ctas = j->op->g.ntiles * 4;
   j->eng.external = sv->cfg.batching >= 0 && ctas <= BATCH_MAX_CTAS;
   if ((st = engine_start(&j->eng))) return st;

@@ -68,9 +68,9 @@ struct SolverEngine {
 size_t solve_ws_layout(const mf_operator* op, int mixed, char* base, SolveWs* w);
 
 // A continuous batch of CG solves of one class (degree, path, kind, vector element type and
-// launch variant): descriptors of all members in device memory, and the CTA counts of the
+// launch configuration): descriptors of all members in device memory, and the CTA counts of the
 // batched launches.  batch_plan_build stages the descriptors in host (pinned) memory and
-// copies them on stream s; batch_iteration enqueues one CG iteration of every member (four
+// copies them on stream s; batch_iteration enqueues one CG iteration of every member (three
 // launches); batch_gather_states copies every member's CgState to states_dev[i].
 struct BatchPlan {
   int n = 0, elem = 0, vk = 0;
