@@ -426,8 +426,8 @@ __global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N)) c
   cg_update_body<T, N>(x, r, p, q, dinv, g, sc, st, hist, partials, nparts, blockIdx.x, gridDim.x);
 }
 // CTAs of an update: one warp per x-pencil unit up to one wave of resident CTAs, whose warps then
-// loop.  Several waves each
-// paid the launch and the reduction's tail (Q4 FP32 24^3, L2-resident: see cg_update_body's use).
+// loop.  Several waves each paid the launch and the reduction's tail: with the folded alpha, a CG
+// iteration of Q4 FP32 on 24^3 (vectors in L2) went from 46.7 to 36.7 us, FP64 103.9 to 89.6.
 static int update_ctas(const mf_operator* op, int elem) {
   const long long units = op->g.ntiles * op->n * op->n, need = (units + RED_THREADS / 32 - 1) / (RED_THREADS / 32);
   const int wave = 152 * update_minb(elem == 4, op->n);
