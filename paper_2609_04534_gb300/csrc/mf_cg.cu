@@ -281,10 +281,12 @@ __global__ void cg_p_kernel(const T* __restrict__ r, T* __restrict__ p, const fl
 // x-neighbours at both pencil ends) is issued before any sum, so a thread keeps up to 7n + 8
 // loads in flight.
 // With nparts > 0 the kernel first folds the apply's nparts partials of <p, A p> itself, every
-// CTA the same sum in the same order, and forms alpha = <r, z> / <p, A p> (breakdown when the
-// sum is not positive and finite; CTA 0 records it); otherwise alpha is in the state.  A separate
-// one-CTA kernel for it costs 4 us and a launch gap, a large part of an iteration of a small
-// problem.
+// CTA the same sum in the same order, and forms alpha = <r, z> / <p, A p>; otherwise alpha is in
+// the state.  A separate one-CTA kernel for it costs 4 us and a launch gap, a large part of an
+// iteration of a small problem.  On breakdown (the sum is not positive and finite, in every CTA
+// alike) no CTA touches x or r.  Every CTA reads the state before it takes its ticket of the
+// final reduction, and only the last one to take a ticket writes it, so the state does not change
+// while a CTA may read it.
 template <typename T, int N>
 __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
                                                const T* __restrict__ q, const float* __restrict__ dinv,
@@ -296,21 +298,15 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
     for (int i = threadIdx.x; i < nparts; i += RED_THREADS) pq += partials[i];
   }
   if (st->flag != 0) return; // uniform: converged or stopped, nothing changes
+  bool broken = false;
   if (nparts > 0) {
     __shared__ double s_pq;
     pq = block_sum(pq);
     if (threadIdx.x == 0) s_pq = pq;
     __syncthreads();
     pq = s_pq;
-    if (!(pq > 0.0) || !isfinite(pq)) {
-      if (cta == 0 && threadIdx.x == 0) {
-        st->pq = pq;
-        st->alpha = 0.0;
-        st->flag = 2; // a CTA that starts later sees it and returns, as it would by the sum
-      }
-      return;
-    }
-    alpha = st->rz / pq;
+    broken = !(pq > 0.0) || !isfinite(pq);
+    alpha = broken ? 0.0 : st->rz / pq;
   }
   const T al = scalar_from_double<T>(alpha);
   const long long tile_el = (long long)N3 * BL;                 // elements of one tile
@@ -329,7 +325,7 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
   // 32-bit: a unit is 32 n elements of a vector that fits the device
   const int units = (int)(g.ntiles * N2), warps = ncta * (RED_THREADS / 32), txy = g.ntx * g.nty;
   typename AccOf<T>::type acc, accz; // <r, r> and (preconditioned) <r, z>
-  for (int u = cta * (RED_THREADS / 32) + (threadIdx.x >> 5); u < units; u += warps) {
+  for (int u = broken ? units : cta * (RED_THREADS / 32) + (threadIdx.x >> 5); u < units; u += warps) {
     const int t = u / N2;
     const int jk = u - t * N2;
     const int j = jk % N, k = jk / N;
@@ -399,6 +395,12 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
   const double sz = dinv ? block_sum(accz.value()) : 0.0;
   double tot, totz;
   if (last_block_total2(sc, s, sz, &tot, &totz, cta, ncta)) {
+    if (broken) {
+      st->pq = pq;
+      st->alpha = 0.0;
+      st->flag = 2;
+      return;
+    }
     const double rz = dinv ? totz : tot;
     st->beta = rz / st->rz;
     st->rz = rz;
