@@ -226,15 +226,15 @@ struct alignas(4 * sizeof(T) < 16 ? 16 : 4 * sizeof(T)) Quad {
 // p = r + beta p, two quads per thread and trip so that four 16-byte loads are in flight
 // p = z + beta p, z = r or, with dinv, z = r / diag(A)
 template <typename T>
-__device__ __forceinline__ void cg_p_body(const T* __restrict__ r, T* __restrict__ p, const float* __restrict__ dinv,
-                                          long long n, const CgState* st, long long cta, long long ncta) {
+__device__ __forceinline__ void cg_p_body(const T* r, T* p, const float* __restrict__ dinv, long long n,
+                                          const CgState* st, long long cta, long long ncta) {
   const T be = scalar_from_double<T>(st->beta);
   // stopped (converged, broken down or at maxit): the direction stays the last one applied,
   // which a reliable update of the mixed solver continues from
   if (st->flag != 0) return;
   const long long nq = n / 4;
-  const Quad<T>* __restrict__ rq = reinterpret_cast<const Quad<T>*>(r);
-  Quad<T>* __restrict__ pq = reinterpret_cast<Quad<T>*>(p);
+  const Quad<T>* rq = reinterpret_cast<const Quad<T>*>(r);
+  Quad<T>* pq = reinterpret_cast<Quad<T>*>(p);
   const long long stride = ncta * blockDim.x;
   for (long long i = cta * (long long)blockDim.x + threadIdx.x; i < nq; i += 2 * stride) {
     const bool two = i + stride < nq;
@@ -261,8 +261,7 @@ __device__ __forceinline__ void cg_p_body(const T* __restrict__ r, T* __restrict
   }
 }
 template <typename T>
-__global__ void cg_p_kernel(const T* __restrict__ r, T* __restrict__ p, const float* __restrict__ dinv, long long n,
-                            const CgState* st) {
+__global__ void cg_p_kernel(const T* r, T* p, const float* __restrict__ dinv, long long n, const CgState* st) {
   pdl_enter();
   cg_p_body<T>(r, p, dinv, n, st, blockIdx.x, gridDim.x);
 }
@@ -288,10 +287,9 @@ __global__ void cg_p_kernel(const T* __restrict__ r, T* __restrict__ p, const fl
 // final reduction, and only the last one to take a ticket writes it, so the state does not change
 // while a CTA may read it.
 template <typename T, int N>
-__device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
-                                               const T* __restrict__ q, const float* __restrict__ dinv,
+__device__ __forceinline__ void cg_update_body(T* x, T* r, const T* p, const T* q, const float* __restrict__ dinv,
                                                const GridInfo& g, RedScratch* sc, CgState* st, double* hist,
-                                               const double* __restrict__ partials, int nparts, int cta, int ncta) {
+                                               const double* partials, int nparts, int cta, int ncta) {
   constexpr int N2 = N * N, N3 = N2 * N, K = N - 1;
   double alpha = st->alpha, pq = 0.0;
   if (nparts > 0) {
@@ -419,11 +417,9 @@ __device__ __forceinline__ void cg_update_body(T* __restrict__ x, T* __restrict_
 // CTAs per SM of the update by registers: a lane's loads in flight grow with n.
 constexpr int update_minb(bool f32, int n) { return f32 ? (n <= 6 ? 3 : 2) : (n <= 7 ? 2 : 1); }
 template <typename T, int N>
-__global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N)) cg_update_kernel(T* __restrict__ x, T* __restrict__ r,
-                                                                const T* __restrict__ p, const T* __restrict__ q,
-                                                                const float* __restrict__ dinv, GridInfo g,
-                                                                RedScratch* sc, CgState* st, double* hist,
-                                                                const double* __restrict__ partials, int nparts) {
+__global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N))
+    cg_update_kernel(T* x, T* r, const T* p, const T* q, const float* __restrict__ dinv, GridInfo g, RedScratch* sc,
+                     CgState* st, double* hist, const double* partials, int nparts) {
   pdl_enter();
   cg_update_body<T, N>(x, r, p, q, dinv, g, sc, st, hist, partials, nparts, blockIdx.x, gridDim.x);
 }
@@ -440,7 +436,7 @@ constexpr long long UPDATE_FOLD_MAX = 16384;
 
 // alpha = <r, r> / <p, A p> from the apply's per-CTA partials of <p, A p>, folded in a fixed
 // order (breakdown when <p, A p> is not positive and finite).
-__device__ __forceinline__ void alpha_body(const double* __restrict__ partials, long long nparts, CgState* st) {
+__device__ __forceinline__ void alpha_body(const double* partials, long long nparts, CgState* st) {
   __shared__ double park[1024];
   if (st->flag != 0) return; // uniform
   double s = 0.0;

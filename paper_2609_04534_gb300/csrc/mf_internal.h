@@ -109,8 +109,8 @@ struct CgFuse {
 // same degree shares them in its parameters).
 template <typename S, typename T>
 struct ApplyJob {
-  const S* __restrict__ x;
-  S* __restrict__ y;
+  const S* x;
+  S* y;
   const T* __restrict__ geom; // curved: [tile][comp][l][lane], 6 (Laplace) or 7 (Helmholtz) comps
   GridInfo g;
   T G[6];                     // affine: w-free metric w det J J^-1 J^-T (xx,xy,xz,yy,yz,zz)

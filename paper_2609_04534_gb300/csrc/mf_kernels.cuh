@@ -186,6 +186,39 @@ __device__ __forceinline__ T load_value(S v) {
     return to_compute<T, S>(v);
 }
 
+// N values of the input from element e0, `step` elements apart, of one cell (CPL = 1; real: v0) or a
+// pair (CPL = 2, 8-byte accesses; real: v0, v1): x, or in a CG step with update_p the new
+// direction p = r + beta p, written back (zero in padding cells).  Every load is issued before the
+// first store, which the compiler must assume to change what a later load reads (mf_launch.cuh).
+template <typename S, int CPL, int N>
+struct LoadLine {
+  typename std::conditional<CPL == 2, float2, S>::type x[N];
+  template <typename T>
+  __device__ __forceinline__ LoadLine(const ApplyJob<S, T>& a, bool fuse, S beta, long long e0, int step, bool v0,
+                                      bool v1) {
+    using V = typename std::conditional<CPL == 2, float2, S>::type;
+    const S* src = fuse ? a.cg.p : a.x;
+#pragma unroll
+    for (int m = 0; m < N; ++m)
+      if (CPL == 2 || v0) x[m] = *reinterpret_cast<const V*>(src + e0 + (long long)m * step);
+    if (!fuse) return;
+    V r[N];
+#pragma unroll
+    for (int m = 0; m < N; ++m)
+      if (CPL == 2 || v0) r[m] = *reinterpret_cast<const V*>(a.cg.r + e0 + (long long)m * step);
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+      if constexpr (CPL == 2) {
+        x[m].x = v0 ? fmaf(beta, x[m].x, r[m].x) : 0.0f;
+        x[m].y = v1 ? fmaf(beta, x[m].y, r[m].y) : 0.0f;
+      } else {
+        x[m] = v0 ? finish(fma(beta, x[m], r[m])) : S(0);
+      }
+      *reinterpret_cast<V*>(a.cg.p + e0 + (long long)m * step) = x[m];
+    }
+  }
+};
+
 // Load the CB values (CB * CPL cells from lane0) of tile t into smem as buf[l*CB + c] (cell
 // fastest; a pair value holds cells lane0 + 2c and lane0 + 2c + 1), zeroing padding cells and,
 // for Dirichlet, the constrained nodes (the P of P A P).  In a CG step with update_p the loaded
@@ -199,47 +232,28 @@ __device__ __forceinline__ void load_tile(const ApplyJob<S, T>& a, long long t, 
   const long long base = t * (long long)N3 * BL + lane0;
   const bool fuse = a.cg.st != nullptr && a.cg.update_p;
   const S beta = fuse ? scalar_from_double<S>(a.cg.st->beta) : S(0);
-  S* __restrict__ pg = a.cg.p;
-  const S* __restrict__ rg = a.cg.r;
   const int c = threadIdx.x % CB, l0 = threadIdx.x / CB;
+  const long long e0 = base + (long long)l0 * BL + c * CPL; // local dof l0 + m n^2 at e0 + m n^2 BL
   int cx, cy, cz;
   cell_of(a.g, t, lane0 + c * CPL, cx, cy, cz); // for a pair: the second cell is at cx + 1
+  const bool yz = cy < a.g.ny && cz < a.g.nz;
+  const bool v0 = yz && cx < a.g.nx, v1 = yz && cx + 1 < a.g.nx;
+  LoadLine<S, CPL, N> in(a, fuse, beta, e0, N2 * BL, v0, v1);
 #pragma unroll
   for (int m = 0; m < N; ++m) {
     const int l = l0 + m * N2, idx = l * CB + c;
-    const long long e = base + (long long)l * BL + c * CPL;
     if constexpr (CPL == 1) {
       T v = T(0);
-      if (cx < a.g.nx && cy < a.g.ny && cz < a.g.nz) {
-        S xv;
-        if (fuse) {
-          xv = finish(fma(beta, pg[e], rg[e]));
-          pg[e] = xv;
-        } else {
-          xv = a.x[e];
-        }
-        v = load_value<INL, (N >= 4), T, S>(xv);
+      if (v0) {
+        v = load_value<INL, (N >= 4), T, S>(in.x[m]);
         if (a.g.bc) {
           const int i = l % N, j = (l / N) % N, k = l / N2;
           if (on_cube_boundary<N>(a.g, cx, cy, cz, i, j, k)) v = T(0);
         }
-      } else if (fuse) {
-        pg[e] = S(0);
       }
       buf[idx] = v;
     } else { // a pair of cells (FP32): 8-byte accesses
-      const bool yz = cy < a.g.ny && cz < a.g.nz;
-      const bool v0 = yz && cx < a.g.nx, v1 = yz && cx + 1 < a.g.nx;
-      float2 xv;
-      if (fuse) {
-        const float2 pv = *reinterpret_cast<const float2*>(pg + e);
-        const float2 rv = *reinterpret_cast<const float2*>(rg + e);
-        xv.x = v0 ? fmaf(beta, pv.x, rv.x) : 0.0f;
-        xv.y = v1 ? fmaf(beta, pv.y, rv.y) : 0.0f;
-        *reinterpret_cast<float2*>(pg + e) = xv;
-      } else {
-        xv = *reinterpret_cast<const float2*>(a.x + e);
-      }
+      const float2 xv = in.x[m];
       float vx = v0 ? xv.x : 0.0f, vy = v1 ? xv.y : 0.0f;
       if (a.g.bc) {
         const int i = l % N, j = (l / N) % N, k = l / N2;
@@ -261,47 +275,25 @@ __device__ __forceinline__ void load_xpencil(const ApplyJob<S, T>& a, long long 
   const long long base = t * (long long)N3 * BL + lane0 + c * CPL;
   const bool fuse = a.cg.st != nullptr && a.cg.update_p;
   const S beta = fuse ? scalar_from_double<S>(a.cg.st->beta) : S(0);
-  S* __restrict__ pg = a.cg.p;
-  const S* __restrict__ rg = a.cg.r;
   int cx, cy, cz;
   cell_of(a.g, t, lane0 + c * CPL, cx, cy, cz); // for a pair: the second cell is at cx + 1
+  const bool yz = cy < a.g.ny && cz < a.g.nz;
+  const bool v0 = yz && cx < a.g.nx, v1 = yz && cx + 1 < a.g.nx;
+  LoadLine<S, CPL, N> ld(a, fuse, beta, base + (long long)(N * j + N2 * k) * BL, BL, v0, v1);
   if constexpr (CPL == 1) {
-    const bool valid = cx < a.g.nx && cy < a.g.ny && cz < a.g.nz;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const long long e = base + (long long)(i + N * j + N2 * k) * BL;
       T v = T(0);
-      if (valid) {
-        S xv;
-        if (fuse) {
-          xv = finish(fma(beta, pg[e], rg[e]));
-          pg[e] = xv;
-        } else {
-          xv = a.x[e];
-        }
-        v = load_value<InlineFrom<N>::cartesian, (N >= 4), T, S>(xv);
+      if (v0) {
+        v = load_value<InlineFrom<N>::cartesian, (N >= 4), T, S>(ld.x[i]);
         if (a.g.bc && on_cube_boundary<N>(a.g, cx, cy, cz, i, j, k)) v = T(0);
-      } else if (fuse) {
-        pg[e] = S(0);
       }
       in[i] = v;
     }
   } else {
-    const bool yz = cy < a.g.ny && cz < a.g.nz;
-    const bool v0 = yz && cx < a.g.nx, v1 = yz && cx + 1 < a.g.nx;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const long long e = base + (long long)(i + N * j + N2 * k) * BL;
-      float2 xv;
-      if (fuse) {
-        const float2 pv = *reinterpret_cast<const float2*>(pg + e);
-        const float2 rv = *reinterpret_cast<const float2*>(rg + e);
-        xv.x = v0 ? fmaf(beta, pv.x, rv.x) : 0.0f;
-        xv.y = v1 ? fmaf(beta, pv.y, rv.y) : 0.0f;
-        *reinterpret_cast<float2*>(pg + e) = xv;
-      } else {
-        xv = *reinterpret_cast<const float2*>(a.x + e);
-      }
+      const float2 xv = ld.x[i];
       float vx = v0 ? xv.x : 0.0f, vy = v1 ? xv.y : 0.0f;
       if (a.g.bc) {
         if (v0 && on_cube_boundary<N>(a.g, cx, cy, cz, i, j, k)) vx = 0.0f;
@@ -449,7 +441,7 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
     constexpr int CPL = CellsPer<T>::value;
     S pv[N * CPL];
     if (a.cg.st != nullptr) {
-      const S* __restrict__ pg = (a.cg.update_p ? a.cg.p : a.x) + t * (long long)N3 * BL + lane0 + c * CPL;
+      const S* pg = (a.cg.update_p ? a.cg.p : a.x) + t * (long long)N3 * BL + lane0 + c * CPL;
 #pragma unroll
       for (int i = 0; i < N; ++i)
 #pragma unroll
@@ -573,7 +565,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
     constexpr int CPL = CellsPer<T>::value;
     S pv[N * CPL];
     if (a.cg.st != nullptr) {
-      const S* __restrict__ pg = (a.cg.update_p ? a.cg.p : a.x) + t * (long long)N3 * BL + lane0 + c * CPL;
+      const S* pg = (a.cg.update_p ? a.cg.p : a.x) + t * (long long)N3 * BL + lane0 + c * CPL;
 #pragma unroll
       for (int i = 0; i < N; ++i)
 #pragma unroll
@@ -1025,7 +1017,7 @@ struct DssLane {
 // `count` (<= U) rows of one kind (A / B / C: on the high x / y / z face of the cell), ST
 // elements apart from y[0]; low: the rows lie on a low mesh face.
 template <typename T, bool A, bool B, bool C, int U, int ST>
-__device__ __forceinline__ void dss_rows(T* __restrict__ y, const DssLane& d, int count, bool low) {
+__device__ __forceinline__ void dss_rows(T* y, const DssLane& d, int count, bool low) {
   const bool X = A && d.h[0], Y = B && d.h[1], Z = C && d.h[2];
   const bool zero = d.mask && (low || (A && !X) || (B && !Y) || (C && !Z));
   if (!(X || Y || Z || zero)) return;
@@ -1083,8 +1075,7 @@ __device__ __forceinline__ void dss_rows(T* __restrict__ y, const DssLane& d, in
 // Warp u of the launch: chunk u % CHUNKS of tile u / CHUNKS for u < nmain, then row by row the
 // LOW rows of the low-face tiles (the layer tz = 0, then ty = 0, then tx = 0 of the rest).
 template <typename T, int N>
-__global__ void __launch_bounds__(DSS_THREADS) dss_kernel(T* __restrict__ y, GridInfo g, int avg, long long nmain,
-                                                          long long nunits) {
+__global__ void __launch_bounds__(DSS_THREADS) dss_kernel(T* y, GridInfo g, int avg, long long nmain, long long nunits) {
   using D = DssCfg<N>;
   constexpr int K = N - 1, N2 = N * N, N3 = N2 * N, U = D::U, CL = D::CL, E1 = D::E > 0 ? D::E : 1;
   pdl_enter();

@@ -92,18 +92,28 @@ __device__ __forceinline__ void load_plane(const ApplyJob<S, T>& a, const PlaneC
     const PlaneMask<N> m(a.g, q.cx, q.cy, q.cz, k);
     S x[N][N];
     if (fuse) {
-      S* __restrict__ pg = a.cg.p + base;
-      const S* __restrict__ rg = a.cg.r + base;
+      S* pg = a.cg.p + base;
+      const S* rg = a.cg.r + base;
+      S r[N][N]; // every load before the first store (see LoadLine)
 #pragma unroll
       for (int j = 0; j < N; ++j)
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          x[j][i] = S(0);
-          if (q.v0) x[j][i] = finish(fma(beta, pg[(i + N * j) * BL], rg[(i + N * j) * BL]));
+          x[j][i] = r[j][i] = S(0);
+          if (q.v0) {
+            x[j][i] = pg[(i + N * j) * BL];
+            r[j][i] = rg[(i + N * j) * BL];
+          }
+        }
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          x[j][i] = q.v0 ? finish(fma(beta, x[j][i], r[j][i])) : S(0);
           if (in) pg[(i + N * j) * BL] = x[j][i];
         }
     } else {
-      const S* __restrict__ xg = a.x + base;
+      const S* xg = a.x + base;
 #pragma unroll
       for (int j = 0; j < N; ++j)
 #pragma unroll
@@ -126,24 +136,33 @@ __device__ __forceinline__ void load_plane(const ApplyJob<S, T>& a, const PlaneC
   } else {
     const PlaneMask<N> m0(a.g, q.cx, q.cy, q.cz, k), m1(a.g, q.cx + 1, q.cy, q.cz, k);
     float2 x[N][N];
-    if (fuse) {
-      S* __restrict__ pg = a.cg.p + base;
-      const S* __restrict__ rg = a.cg.r + base;
-#pragma unroll
-      for (int j = 0; j < N; ++j)
+    if (fuse) { // row by row, a row's loads before the stores of the row before it (see LoadLine)
+      S* pg = a.cg.p + base;
+      const S* rg = a.cg.r + base;
+      float2 r[2][N];
+      auto load_row = [&](int j) {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          float2 pv = make_float2(0.f, 0.f), rv = pv;
+          x[j][i] = r[j & 1][i] = make_float2(0.f, 0.f);
           if (in) {
-            pv = *reinterpret_cast<const float2*>(pg + (i + N * j) * BL);
-            rv = *reinterpret_cast<const float2*>(rg + (i + N * j) * BL);
+            x[j][i] = *reinterpret_cast<const float2*>(pg + (i + N * j) * BL);
+            r[j & 1][i] = *reinterpret_cast<const float2*>(rg + (i + N * j) * BL);
           }
-          x[j][i].x = q.v0 ? fmaf(beta, pv.x, rv.x) : 0.0f;
-          x[j][i].y = q.v1 ? fmaf(beta, pv.y, rv.y) : 0.0f;
+        }
+      };
+      load_row(0);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        if (j + 1 < N) load_row(j + 1);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          x[j][i].x = q.v0 ? fmaf(beta, x[j][i].x, r[j & 1][i].x) : 0.0f;
+          x[j][i].y = q.v1 ? fmaf(beta, x[j][i].y, r[j & 1][i].y) : 0.0f;
           if (in) *reinterpret_cast<float2*>(pg + (i + N * j) * BL) = x[j][i];
         }
+      }
     } else {
-      const S* __restrict__ xg = a.x + base;
+      const S* xg = a.x + base;
 #pragma unroll
       for (int j = 0; j < N; ++j)
 #pragma unroll
@@ -175,38 +194,50 @@ __device__ __forceinline__ double store_plane(const ApplyJob<S, T>& a, const Pla
   constexpr int N2 = N * N, N3 = N2 * N, CPL = CellsPer<T>::value;
   if (q.t >= a.g.ntiles) return 0.0;
   const long long base = (q.t * N3 + (long long)N2 * k) * BL + q.lane;
-  S* __restrict__ yg = a.y + base;
+  S* yg = a.y + base;
   typename AccOf<S>::type acc;
   const bool pair = PAIR && a.cg.st != nullptr;
-  const S* __restrict__ pg = pair ? (a.cg.update_p ? a.cg.p : a.x) + base : nullptr;
+  const S* pg = pair ? (a.cg.update_p ? a.cg.p : a.x) + base : nullptr;
   if constexpr (CPL == 1) {
     const PlaneMask<N> m(a.g, q.cx, q.cy, q.cz, k);
+    auto value = [&](int j, int i) {
+      const S v = q.v0 ? to_storage<S, T>(u[j][i]) : S(0);
+      return m.on && m(i, j) ? S(0) : v;
+    };
+    if (pair && q.v0) { // its loads before the first store (see LoadLine)
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc.add(pg[(i + N * j) * BL], value(j, i));
+    }
 #pragma unroll
     for (int j = 0; j < N; ++j)
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        S v = q.v0 ? to_storage<S, T>(u[j][i]) : S(0);
-        if (m.on && m(i, j)) v = S(0);
-        yg[(i + N * j) * BL] = v;
-        if (pair && q.v0) acc.add(pg[(i + N * j) * BL], v);
-      }
+      for (int i = 0; i < N; ++i) yg[(i + N * j) * BL] = value(j, i);
   } else {
     const PlaneMask<N> m0(a.g, q.cx, q.cy, q.cz, k), m1(a.g, q.cx + 1, q.cy, q.cz, k);
+    auto value = [&](int j, int i) {
+      float2 v = make_float2(q.v0 ? u[j][i].x : 0.0f, q.v1 ? u[j][i].y : 0.0f);
+      if (m0.on) {
+        if (m0(i, j)) v.x = 0.0f;
+        if (m1(i, j)) v.y = 0.0f;
+      }
+      return v;
+    };
+    if (pair) {
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const float2 pv = *reinterpret_cast<const float2*>(pg + (i + N * j) * BL), v = value(j, i);
+          if (q.v0) acc.add(pv.x, v.x);
+          if (q.v1) acc.add(pv.y, v.y);
+        }
+    }
 #pragma unroll
     for (int j = 0; j < N; ++j)
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        float2 v = make_float2(q.v0 ? u[j][i].x : 0.0f, q.v1 ? u[j][i].y : 0.0f);
-        if (m0.on) {
-          if (m0(i, j)) v.x = 0.0f;
-          if (m1(i, j)) v.y = 0.0f;
-        }
-        *reinterpret_cast<float2*>(yg + (i + N * j) * BL) = v;
-        if (pair) {
-          if (q.v0) acc.add(pg[(i + N * j) * BL], v.x);
-          if (q.v1) acc.add(pg[(i + N * j) * BL + 1], v.y);
-        }
-      }
+      for (int i = 0; i < N; ++i) *reinterpret_cast<float2*>(yg + (i + N * j) * BL) = value(j, i);
   }
   return pair ? acc.value() : 0.0;
 }

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(TC_NT, 1) apply_cartesian_tc(const __grid_cons
     long long t;
     int cx, cy, cz;
     const bool valid = tc_cell(a.g, gp, c, t, cx, cy, cz);
-    double* __restrict__ yp = a.y + t * (long long)NN * BL + (c & 31);
+    double* yp = a.y + t * (long long)NN * BL + (c & 31);
     {
       uint32_t r[TC_S][CH];
 #pragma unroll
