@@ -61,11 +61,9 @@ __device__ __forceinline__ dd fma(dd a, dd b, dd c) {
 
 // The same in 10 instructions instead of 12, for chains of up to three terms: TwoSum's last
 // difference p - v and TwoProd's error a.hi b.hi - p are taken together, as a.hi b.hi - v in one
-// fma, and the cross terms go straight into lo.  lo is rounded once more per term, which shows in long
-// chains (relative error of the Cartesian apply against 64 bits, n = 7, 8: 1.06-1.11 times that of
-// fma(); n <= 5: 0.94-1.04), so it is used by kernels of n <= 5 and by the forward sweeps of the
-// Cartesian kernel at n = 6..8, where the rounded conversion of the input outweighs it (split apply,
-// FP64: Q4 curved 52^3 0.537 -> 0.509 ms, Q4 Cartesian 52^3 0.226 -> 0.212, Q2 curved 88^3 0.409 -> 0.387).
+// fma, and the cross terms go straight into lo.  lo is rounded once more per term, so it is used
+// only where the rounded conversion of double input outweighs that (ShortProducts, mf_kernels.cuh; split
+// apply, FP64: Q4 curved 52^3 0.537 -> 0.509 ms, Q4 Cartesian 52^3 0.226 -> 0.212).
 __device__ __forceinline__ dd fma_short(dd a, dd b, dd c) {
   const float p = a.hi * b.hi;
   const float s = __fadd_rn(c.hi, p);

@@ -133,6 +133,18 @@ __device__ __forceinline__ double sub_lazy(double a, double b) { return a - b; }
 __device__ __forceinline__ float add_lazy(float a, float b) { return a + b; }
 __device__ __forceinline__ float sub_lazy(float a, float b) { return a - b; }
 
+// Where double-float products take the form of 10 instructions (fma_short): only where double
+// input is converted with rounding, which outweighs their extra rounding -- n = 4, 5, and the
+// forward sweeps of the Cartesian kernels to n = 8.  Vectors kept in double-float (CG) convert
+// nothing, and at n = 2, 3 the conversion truncates.  Relative error against 64 bits over that
+// with fma() everywhere and truncated conversion (L2, three inputs, 10^3 to 44^3 cells): applies at
+// n >= 4 0.89-1.00; with fma_short at n = 3 too 1.00-1.01 there, and in CG 1.01-1.04.
+template <typename S, typename T, int N>
+struct ShortProducts {
+  static constexpr bool rounded = std::is_same<S, double>::value && std::is_same<T, dd>::value && N >= 4;
+  static constexpr bool all = rounded && N <= 5, forward = rounded && N <= 8;
+};
+
 // sum_i c[i] x[i], i < M (M >= 1), not renormalised
 template <typename C, typename T, bool SHORT, int M>
 __device__ __forceinline__ T chain(const C* c, const T* x) {
@@ -147,7 +159,7 @@ __device__ __forceinline__ f2 sub_lazy(f2 a, f2 b) { return a + (-b); }
 // Even-odd 1D contraction of one pencil (see EoTab): the pencil folded into its sum and
 // difference halves, H (H + 1) products per half instead of n^2 in all.  ANTI: the matrix is
 // centro-antisymmetric.  out[q] finished.
-template <typename T, int N, bool ANTI>
+template <typename T, int N, bool ANTI, bool SHORT = false>
 struct Fold {
   static constexpr int H = N / 2, HE = (N + 1) / 2;
   T e[HE], o[H > 0 ? H : 1];
@@ -163,12 +175,12 @@ struct Fold {
   __device__ __forceinline__ void apply(const EoTab<C, N>& t, T* out) const {
 #pragma unroll
     for (int q = 0; q < H; ++q) {
-      const T u = chain<C, T, (N <= 5), HE>(t.F + q * HE, e);
-      const T w = chain<C, T, (N <= 5), H>(t.G + q * H, o);
+      const T u = chain<C, T, SHORT, HE>(t.F + q * HE, e);
+      const T w = chain<C, T, SHORT, H>(t.G + q * H, o);
       out[q] = finish(add_lazy(u, w));
       out[N - 1 - q] = finish(ANTI ? sub_lazy(w, u) : sub_lazy(u, w));
     }
-    if (N % 2) out[H] = finish(ANTI ? chain<C, T, (N <= 5), H>(t.Mid, o) : chain<C, T, (N <= 5), HE>(t.Mid, e));
+    if (N % 2) out[H] = finish(ANTI ? chain<C, T, SHORT, H>(t.Mid, o) : chain<C, T, SHORT, HE>(t.Mid, e));
   }
 };
 
@@ -377,6 +389,7 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
                                                long long t, int lane0,
                                                long long cta) {
   constexpr int N2 = N * N, N3 = N2 * N, NT = N2 * CB;
+  constexpr bool SH = ShortProducts<S, T, N>::all;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf0 = reinterpret_cast<T*>(smem_raw);
   T* buf1 = buf0 + N3 * CB;
@@ -389,7 +402,7 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
     T in[N], mo[N], ko[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) in[i] = buf0[(i + N * pa + N2 * pb) * CB + c];
-    const Fold<T, N, false> f(in);
+    const Fold<T, N, false, SH> f(in);
     f.apply(tab.eM, mo);
     f.apply(tab.eK, ko);
 #pragma unroll
@@ -407,11 +420,11 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
       ak[j] = buf1[(pa + N * j + N2 * pb) * CB + c];
     }
     {
-      const Fold<T, N, false> fa(am);
+      const Fold<T, N, false, SH> fa(am);
       fa.apply(tab.eM, mm);
       fa.apply(tab.eK, km);
     }
-    Fold<T, N, false>(ak).apply(tab.eM, mk);
+    Fold<T, N, false, SH>(ak).apply(tab.eM, mk);
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       T w = fma(a.gx, mk[q], mul0(a.gy, km[q]));
@@ -428,8 +441,8 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
       w[k] = buf0[(pa + N * pb + N2 * k) * CB + c];
       mm[k] = buf1[(pa + N * pb + N2 * k) * CB + c];
     }
-    Fold<T, N, false>(w).apply(tab.eM, so);
-    Fold<T, N, false>(mm).apply(tab.eK, ro);
+    Fold<T, N, false, SH>(w).apply(tab.eM, so);
+    Fold<T, N, false, SH>(mm).apply(tab.eK, ro);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < N; ++q) buf0[(pa + N * pb + N2 * q) * CB + c] = finish(fma(a.gz, ro[q], so[q]));
@@ -469,27 +482,27 @@ __device__ __forceinline__ void cartesian_body(const ApplyJob<S, T>& a, const Ta
 // seven, and the pointwise scale replaces the combination of the contractions.
 // ---------------------------------------------------------------------------------------
 // forward: modes of a pencil (symmetric first), from its folded sums and differences
-template <typename C, typename T, int N>
+template <bool SHORT, typename C, typename T, int N>
 __device__ __forceinline__ void fd_forward(const FdTab<C, N>& t, const T* in, T* out) {
   constexpr int H = N / 2, HE = (N + 1) / 2;
   const Fold<T, N, false> f(in);
 #pragma unroll
-  for (int m = 0; m < HE; ++m) out[m] = finish(chain<C, T, (N <= 8), HE>(t.Ff + m * HE, f.e));
+  for (int m = 0; m < HE; ++m) out[m] = finish(chain<C, T, SHORT, HE>(t.Ff + m * HE, f.e));
 #pragma unroll
-  for (int m = 0; m < H; ++m) out[HE + m] = finish(chain<C, T, (N <= 8), H>(t.Gf + m * H, f.o));
+  for (int m = 0; m < H; ++m) out[HE + m] = finish(chain<C, T, SHORT, H>(t.Gf + m * H, f.o));
 }
 // backward: nodal values of a pencil from its modes
-template <typename C, typename T, int N>
+template <bool SHORT, typename C, typename T, int N>
 __device__ __forceinline__ void fd_backward(const FdTab<C, N>& t, const T* z, T* out) {
   constexpr int H = N / 2, HE = (N + 1) / 2;
 #pragma unroll
   for (int j = 0; j < H; ++j) {
-    const T u = chain<C, T, (N <= 5), HE>(t.Fb + j * HE, z);
-    const T v = chain<C, T, (N <= 5), H>(t.Gb + j * H, z + HE);
+    const T u = chain<C, T, SHORT, HE>(t.Fb + j * HE, z);
+    const T v = chain<C, T, SHORT, H>(t.Gb + j * H, z + HE);
     out[j] = finish(add_lazy(u, v));
     out[N - 1 - j] = finish(sub_lazy(u, v));
   }
-  if (N % 2) out[H] = finish(chain<C, T, (N <= 5), HE>(t.Fb + H * HE, z));
+  if (N % 2) out[H] = finish(chain<C, T, SHORT, HE>(t.Fb + H * HE, z));
 }
 
 template <typename S, typename T, int N, int CB, bool HELM>
@@ -497,6 +510,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
                                                   long long t, int lane0, long long cta) {
   using C = typename CoefOf<T>::type;
   constexpr int N2 = N * N, N3 = N2 * N, NT = N2 * CB;
+  constexpr bool SH = ShortProducts<S, T, N>::all, SHF = ShortProducts<S, T, N>::forward;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf0 = reinterpret_cast<T*>(smem_raw);
   if (a.cg.st != nullptr && a.cg.st->flag != 0) return; // CG step after convergence: no work
@@ -520,7 +534,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
 #pragma unroll
       for (int i = 0; i < N; ++i) in[i] = buf0[(i + N * pa + N2 * pb) * CB + c];
     }
-    fd_forward<C, T, N>(fd, in, out);
+    fd_forward<SHF, C, T, N>(fd, in, out);
 #pragma unroll
     for (int i = 0; i < N; ++i) buf0[(i + N * pa + N2 * pb) * CB + c] = out[i];
   }
@@ -529,7 +543,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
     T in[N], out[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) in[j] = buf0[(pa + N * j + N2 * pb) * CB + c];
-    fd_forward<C, T, N>(fd, in, out);
+    fd_forward<SHF, C, T, N>(fd, in, out);
 #pragma unroll
     for (int j = 0; j < N; ++j) buf0[(pa + N * j + N2 * pb) * CB + c] = out[j];
   }
@@ -538,7 +552,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
     T in[N], z[N], out[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) in[k] = buf0[(pa + N * pb + N2 * k) * CB + c];
-    fd_forward<C, T, N>(fd, in, z);
+    fd_forward<SHF, C, T, N>(fd, in, z);
     T dxy = fma(fd.lam[pb], a.gy, mul0(fd.lam[pa], a.gx));
     if (HELM) dxy = add_lazy(dxy, a.cmass);
 #pragma unroll
@@ -546,7 +560,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
       const T dk = finish(fma(fd.lam[k], a.gz, dxy));
       z[k] = finish(mul0(dk, z[k]));
     }
-    fd_backward<C, T, N>(fd, z, out);
+    fd_backward<SH, C, T, N>(fd, z, out);
 #pragma unroll
     for (int k = 0; k < N; ++k) buf0[(pa + N * pb + N2 * k) * CB + c] = out[k];
   }
@@ -555,7 +569,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
     T z[N], out[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) z[j] = buf0[(pa + N * j + N2 * pb) * CB + c];
-    fd_backward<C, T, N>(fd, z, out);
+    fd_backward<SH, C, T, N>(fd, z, out);
 #pragma unroll
     for (int j = 0; j < N; ++j) buf0[(pa + N * j + N2 * pb) * CB + c] = out[j];
   }
@@ -574,7 +588,7 @@ __device__ __forceinline__ void cartesian_fd_body(const ApplyJob<S, T>& a, const
     T z[N], o[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) z[i] = buf0[(i + N * pa + N2 * pb) * CB + c];
-    fd_backward<C, T, N>(fd, z, o);
+    fd_backward<SH, C, T, N>(fd, z, o);
     store_xpencil<S, T, N, CB>(a, t, lane0, c, pa, pb, o, acc, pv);
   }
   if (a.cg.st != nullptr) {
@@ -659,6 +673,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
                                              long long cta) {
   constexpr int N2 = N * N, N3 = N2 * N, NT = N2 * CB;
   constexpr int NC = HELM ? 7 : 6;
+  constexpr bool SH = ShortProducts<S, T, N>::all;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf0 = reinterpret_cast<T*>(smem_raw);
   T* buf1 = buf0 + N3 * CB;
@@ -673,7 +688,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N], out[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) in[i] = buf0[(i + N * pa + N2 * pb) * CB + c];
-    Fold<T, N, false>(in).apply(tab.eS, out);
+    Fold<T, N, false, SH>(in).apply(tab.eS, out);
 #pragma unroll
     for (int q = 0; q < N; ++q) buf0[(q + N * pa + N2 * pb) * CB + c] = out[q];
   }
@@ -682,7 +697,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N], out[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) in[j] = buf0[(pa + N * j + N2 * pb) * CB + c];
-    Fold<T, N, false>(in).apply(tab.eS, out);
+    Fold<T, N, false, SH>(in).apply(tab.eS, out);
 #pragma unroll
     for (int q = 0; q < N; ++q) buf0[(pa + N * q + N2 * pb) * CB + c] = out[q];
   }
@@ -694,10 +709,10 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) in[k] = buf0[(pa + N * pb + N2 * k) * CB + c];
-    Fold<T, N, false>(in).apply(tab.eS, U);
+    Fold<T, N, false, SH>(in).apply(tab.eS, U);
 #pragma unroll
     for (int q = 0; q < N; ++q) buf1[(pa + N * pb + N2 * q) * CB + c] = U[q];
-    Fold<T, N, true>(U).apply(tab.eD, d3);
+    Fold<T, N, true, SH>(U).apply(tab.eD, d3);
   }
   __syncthreads();
   { // x- and y-derivatives by Dc, folded like the z one: x-pencil (j=pa, k=pb) of buf1 -> buf0,
@@ -705,12 +720,12 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N], out[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) in[i] = buf1[(i + N * pa + N2 * pb) * CB + c];
-    Fold<T, N, true>(in).apply(tab.eD, out);
+    Fold<T, N, true, SH>(in).apply(tab.eD, out);
 #pragma unroll
     for (int q = 0; q < N; ++q) buf0[(q + N * pa + N2 * pb) * CB + c] = out[q];
 #pragma unroll
     for (int j = 0; j < N; ++j) in[j] = buf1[(pa + N * j + N2 * pb) * CB + c];
-    Fold<T, N, true>(in).apply(tab.eD, out);
+    Fold<T, N, true, SH>(in).apply(tab.eD, out);
 #pragma unroll
     for (int q = 0; q < N; ++q) buf2[(pa + N * q + N2 * pb) * CB + c] = out[q];
   }
@@ -770,9 +785,9 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
         g3 = w * a.G[3]; g4 = w * a.G[4]; g5 = w * a.G[5];
         if (HELM) m = w * a.mdet;
       }
-      v1 = finish(fma_n<(N <= 5)>(g0, d1, fma_n<(N <= 5)>(g1, d2, mul0(g2, d3q))));
-      v2 = finish(fma_n<(N <= 5)>(g1, d1, fma_n<(N <= 5)>(g3, d2, mul0(g4, d3q))));
-      v3 = finish(fma_n<(N <= 5)>(g2, d1, fma_n<(N <= 5)>(g4, d2, mul0(g5, d3q))));
+      v1 = finish(fma_n<SH>(g0, d1, fma_n<SH>(g1, d2, mul0(g2, d3q))));
+      v2 = finish(fma_n<SH>(g1, d1, fma_n<SH>(g3, d2, mul0(g4, d3q))));
+      v3 = finish(fma_n<SH>(g2, d1, fma_n<SH>(g4, d2, mul0(g5, d3q))));
     }
     buf0[l * CB + c] = v1;
     buf2[l * CB + c] = v2;
@@ -789,12 +804,12 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N], out[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) in[q] = buf0[(q + N * pa + N2 * pb) * CB + c];
-    Fold<T, N, true>(in).apply(tab.eDt, out);
+    Fold<T, N, true, SH>(in).apply(tab.eDt, out);
 #pragma unroll
     for (int i = 0; i < N; ++i) buf1[(i + N * pa + N2 * pb) * CB + c] = out[i];
 #pragma unroll
     for (int q = 0; q < N; ++q) in[q] = buf2[(pa + N * q + N2 * pb) * CB + c];
-    Fold<T, N, true>(in).apply(tab.eDt, out);
+    Fold<T, N, true, SH>(in).apply(tab.eDt, out);
 #pragma unroll
     for (int j = 0; j < N; ++j) buf2[(pa + N * j + N2 * pb) * CB + c] = out[j];
   }
@@ -802,7 +817,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
   // t = Dc^T_x v1 (+ m u) + Dc^T_y v2 + Dc^T_z v3 at points (pa, pb, q), then S^T along z
   {
     T tq[N];
-    Fold<T, N, true>(d3).apply(tab.eDt, tq); // Dc^T_z v3 along this pencil
+    Fold<T, N, true, SH>(d3).apply(tab.eDt, tq); // Dc^T_z v3 along this pencil
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       const int l = pa + N * pb + N2 * q;
@@ -811,7 +826,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
       tq[q] = finish(add_lazy(add_lazy(s, buf2[l * CB + c]), tq[q]));
     }
     T out[N];
-    Fold<T, N, false>(tq).apply(tab.eSt, out);
+    Fold<T, N, false, SH>(tq).apply(tab.eSt, out);
 #pragma unroll
     for (int k = 0; k < N; ++k) buf1[(pa + N * pb + N2 * k) * CB + c] = out[k];
   }
@@ -820,7 +835,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N], out[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) in[q] = buf1[(pa + N * q + N2 * pb) * CB + c];
-    Fold<T, N, false>(in).apply(tab.eSt, out);
+    Fold<T, N, false, SH>(in).apply(tab.eSt, out);
 #pragma unroll
     for (int j = 0; j < N; ++j) buf1[(pa + N * j + N2 * pb) * CB + c] = out[j];
   }
@@ -830,7 +845,7 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
     T in[N], o[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) in[q] = buf1[(q + N * pa + N2 * pb) * CB + c];
-    Fold<T, N, false>(in).apply(tab.eSt, o);
+    Fold<T, N, false, SH>(in).apply(tab.eSt, o);
     store_xpencil<S, T, N, CB>(a, t, lane0, c, pa, pb, o, acc, static_cast<const S*>(nullptr));
   }
   if (fuse) { // after the last barrier, so that no warp waits for warp 0's fold

@@ -251,24 +251,24 @@ __device__ __forceinline__ void plane_prefetch(const ApplyJob<S, T>& a, long lon
 }
 
 // A matrix applied to every row (x) or column (y) of a plane, in place.
-template <bool ANTI, typename C, typename T, int N>
+template <bool ANTI, bool SHORT, typename C, typename T, int N>
 __device__ __forceinline__ void plane_x(const EoTab<C, N>& m, T (&u)[N][N]) {
 #pragma unroll
   for (int j = 0; j < N; ++j) {
     T out[N];
-    Fold<T, N, ANTI>(u[j]).apply(m, out);
+    Fold<T, N, ANTI, SHORT>(u[j]).apply(m, out);
 #pragma unroll
     for (int i = 0; i < N; ++i) u[j][i] = out[i];
   }
 }
-template <bool ANTI, typename C, typename T, int N>
+template <bool ANTI, bool SHORT, typename C, typename T, int N>
 __device__ __forceinline__ void plane_y(const EoTab<C, N>& m, T (&u)[N][N]) {
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     T in[N], out[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) in[j] = u[j][i];
-    Fold<T, N, ANTI>(in).apply(m, out);
+    Fold<T, N, ANTI, SHORT>(in).apply(m, out);
 #pragma unroll
     for (int j = 0; j < N; ++j) u[j][i] = out[j];
   }
@@ -282,6 +282,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
                                               long long cta) {
   constexpr int N2 = N * N, N3 = N2 * N, CB = PlaneCfg<T, N>::CB, NT = N * CB, CPL = CellsPer<T>::value;
   constexpr int NC = HELM ? 7 : 6;
+  constexpr bool SH = ShortProducts<S, T, N>::all;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* A = reinterpret_cast<T*>(smem_raw);
   T* B = A + N3 * CB;
@@ -294,8 +295,8 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
   {
     T u[N][N];
     load_plane<false, S, T, N>(a, cell, p, u);
-    plane_x<false>(tab.eS, u);
-    plane_y<false>(tab.eS, u);
+    plane_x<false, SH>(tab.eS, u);
+    plane_y<false, SH>(tab.eS, u);
 #pragma unroll
     for (int j = 0; j < N; ++j)
 #pragma unroll
@@ -307,8 +308,8 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
     T in[N], U[N], d3[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) in[k] = A[(i + N * p + N2 * k) * CB];
-    Fold<T, N, false>(in).apply(tab.eS, U);
-    Fold<T, N, true>(U).apply(tab.eD, d3);
+    Fold<T, N, false, SH>(in).apply(tab.eS, U);
+    Fold<T, N, true, SH>(U).apply(tab.eD, d3);
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       A[(i + N * p + N2 * q) * CB] = U[q];
@@ -324,7 +325,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
     for (int j = 0; j < N; ++j)
 #pragma unroll
       for (int i = 0; i < N; ++i) u[j][i] = d2[j][i] = A[(i + N * j + N2 * p) * CB];
-    plane_y<true>(tab.eD, d2);
+    plane_y<true, SH>(tab.eD, d2);
     float sx[N][2], px[N][2], sz = 0.f, pz = 0.f;
     const float* ty = nullptr;
     if constexpr (CURVED && IsF32<T>::value) { // sin and pi cos of pi xh, see general_body
@@ -349,7 +350,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       T d1[N], mu[N];
-      Fold<T, N, true>(u[j]).apply(tab.eD, d1);
+      Fold<T, N, true, SH>(u[j]).apply(tab.eD, d1);
       float syz = 0.f, pyz = 0.f, spz = 0.f;
       if constexpr (CURVED && IsF32<T>::value) {
         syz = __fmul_rn(ty[2 * j], sz);
@@ -380,9 +381,9 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
             g3 = w * a.G[3]; g4 = w * a.G[4]; g5 = w * a.G[5];
             if (HELM) m = w * a.mdet;
           }
-          v1 = finish(fma_n<(N <= 5)>(g0, e1, fma_n<(N <= 5)>(g1, e2, mul0(g2, e3))));
-          v2 = finish(fma_n<(N <= 5)>(g1, e1, fma_n<(N <= 5)>(g3, e2, mul0(g4, e3))));
-          v3 = finish(fma_n<(N <= 5)>(g2, e1, fma_n<(N <= 5)>(g4, e2, mul0(g5, e3))));
+          v1 = finish(fma_n<SH>(g0, e1, fma_n<SH>(g1, e2, mul0(g2, e3))));
+          v2 = finish(fma_n<SH>(g1, e1, fma_n<SH>(g3, e2, mul0(g4, e3))));
+          v3 = finish(fma_n<SH>(g2, e1, fma_n<SH>(g4, e2, mul0(g5, e3))));
         }
         d1[i] = v1;
         d2[j][i] = v2;
@@ -394,11 +395,11 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
         }
       }
       T out[N];
-      Fold<T, N, true>(d1).apply(tab.eDt, out);
+      Fold<T, N, true, SH>(d1).apply(tab.eDt, out);
 #pragma unroll
       for (int i = 0; i < N; ++i) u[j][i] = HELM ? add_lazy(out[i], mu[i]) : out[i];
     }
-    plane_y<true>(tab.eDt, d2);
+    plane_y<true, SH>(tab.eDt, d2);
 #pragma unroll
     for (int j = 0; j < N; ++j)
 #pragma unroll
@@ -410,10 +411,10 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
     T v3[N], tq[N], out[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) v3[q] = B[(i + N * p + N2 * q) * CB];
-    Fold<T, N, true>(v3).apply(tab.eDt, tq);
+    Fold<T, N, true, SH>(v3).apply(tab.eDt, tq);
 #pragma unroll
     for (int q = 0; q < N; ++q) tq[q] = finish(add_lazy(A[(i + N * p + N2 * q) * CB], tq[q]));
-    Fold<T, N, false>(tq).apply(tab.eSt, out);
+    Fold<T, N, false, SH>(tq).apply(tab.eSt, out);
 #pragma unroll
     for (int k = 0; k < N; ++k) A[(i + N * p + N2 * k) * CB] = out[k];
   }
@@ -424,8 +425,8 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
     for (int j = 0; j < N; ++j)
 #pragma unroll
       for (int i = 0; i < N; ++i) u[j][i] = A[(i + N * j + N2 * p) * CB];
-    plane_y<false>(tab.eSt, u);
-    plane_x<false>(tab.eSt, u);
+    plane_y<false, SH>(tab.eSt, u);
+    plane_x<false, SH>(tab.eSt, u);
     store_plane<false, S, T, N>(a, cell, p, u);
   }
   if (fuse) {
@@ -444,6 +445,7 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
                                                 long long cta) {
   using C = typename CoefOf<T>::type;
   constexpr int N2 = N * N, CB = PlaneCfg<T, N>::CB, NT = N * CB;
+  constexpr bool SH = ShortProducts<S, T, N>::all, SHF = ShortProducts<S, T, N>::forward;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* A = reinterpret_cast<T*>(smem_raw);
   if (a.cg.st != nullptr && a.cg.st->flag != 0) return; // CG step after convergence: no work
@@ -458,7 +460,7 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       T out[N];
-      fd_forward<C, T, N>(fd, u[j], out);
+      fd_forward<SHF, C, T, N>(fd, u[j], out);
 #pragma unroll
       for (int i = 0; i < N; ++i) u[j][i] = out[i];
     }
@@ -467,7 +469,7 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
       T in[N], out[N];
 #pragma unroll
       for (int j = 0; j < N; ++j) in[j] = u[j][i];
-      fd_forward<C, T, N>(fd, in, out);
+      fd_forward<SHF, C, T, N>(fd, in, out);
 #pragma unroll
       for (int j = 0; j < N; ++j) A[(i + N * j + N2 * p) * CB] = out[j];
     }
@@ -478,7 +480,7 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
     T in[N], z[N], out[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) in[k] = A[(i + N * p + N2 * k) * CB];
-    fd_forward<C, T, N>(fd, in, z);
+    fd_forward<SHF, C, T, N>(fd, in, z);
     T dxy = fma(fd.lam[p], a.gy, mul0(fd.lam[i], a.gx));
     if (HELM) dxy = add_lazy(dxy, a.cmass);
 #pragma unroll
@@ -486,7 +488,7 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
       const T dk = finish(fma(fd.lam[k], a.gz, dxy));
       z[k] = finish(mul0(dk, z[k]));
     }
-    fd_backward<C, T, N>(fd, z, out);
+    fd_backward<SH, C, T, N>(fd, z, out);
 #pragma unroll
     for (int k = 0; k < N; ++k) A[(i + N * p + N2 * k) * CB] = out[k];
   }
@@ -499,14 +501,14 @@ __device__ __forceinline__ void cartesian_plane(const ApplyJob<S, T>& a, const T
       T z[N], out[N];
 #pragma unroll
       for (int j = 0; j < N; ++j) z[j] = A[(i + N * j + N2 * p) * CB];
-      fd_backward<C, T, N>(fd, z, out);
+      fd_backward<SH, C, T, N>(fd, z, out);
 #pragma unroll
       for (int j = 0; j < N; ++j) u[j][i] = out[j];
     }
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       T out[N];
-      fd_backward<C, T, N>(fd, u[j], out);
+      fd_backward<SH, C, T, N>(fd, u[j], out);
 #pragma unroll
       for (int i = 0; i < N; ++i) u[j][i] = out[i];
     }
