@@ -156,6 +156,21 @@ __device__ __forceinline__ T chain(const C* c, const T* x) {
 __device__ __forceinline__ f2 add_lazy(f2 a, f2 b) { return a + b; }
 __device__ __forceinline__ f2 sub_lazy(f2 a, f2 b) { return a + (-b); }
 
+// lo = u + w and hi = u - w (ANTI: w - u), w = sum_i c[i] x[i], i < N / 2.  In FP32 at n = 3 the one
+// product goes into the sum by one rounding instead of two (with two, the apply's error against
+// 64 bits was 1.005-1.02 times as large; Fold::add_to does the same).
+template <bool SHORT, int N, bool ANTI, typename C, typename T>
+__device__ __forceinline__ void chain_sum(const C* c, const T* x, T u, T& lo, T& hi) {
+  if constexpr (N == 3 && IsF32<T>::value) {
+    lo = fma(c[0], x[0], u);
+    hi = ANTI ? fma(c[0], x[0], -u) : fma(-c[0], x[0], u);
+  } else {
+    const T w = chain<C, T, SHORT, N / 2>(c, x);
+    lo = add_lazy(u, w);
+    hi = ANTI ? sub_lazy(w, u) : sub_lazy(u, w);
+  }
+}
+
 // Even-odd 1D contraction of one pencil (see EoTab): the pencil folded into its sum and
 // difference halves, H (H + 1) products per half instead of n^2 in all.  ANTI: the matrix is
 // centro-antisymmetric.  out[q] finished.
@@ -176,11 +191,20 @@ struct Fold {
 #pragma unroll
     for (int q = 0; q < H; ++q) {
       const T u = chain<C, T, SHORT, HE>(t.F + q * HE, e);
-      const T w = chain<C, T, SHORT, H>(t.G + q * H, o);
-      out[q] = finish(add_lazy(u, w));
-      out[N - 1 - q] = finish(ANTI ? sub_lazy(w, u) : sub_lazy(u, w));
+      T lo, hi;
+      chain_sum<SHORT, N, ANTI>(t.G + q * H, o, u, lo, hi);
+      out[q] = finish(lo);
+      out[N - 1 - q] = finish(hi);
     }
     if (N % 2) out[H] = finish(ANTI ? chain<C, T, SHORT, H>(t.Mid, o) : chain<C, T, SHORT, HE>(t.Mid, e));
+  }
+  // s + the contraction (in FP32 a row of one product by one rounding, see chain_sum)
+  template <typename C>
+  __device__ __forceinline__ void add_to(const T* s, const EoTab<C, N>& t, T* out) const {
+    apply(t, out);
+#pragma unroll
+    for (int q = 0; q < N; ++q) out[q] = finish(add_lazy(s[q], out[q]));
+    if constexpr (N == 3 && ANTI && IsF32<T>::value) out[1] = fma(t.Mid[0], o[0], s[1]);
   }
 };
 
@@ -498,9 +522,10 @@ __device__ __forceinline__ void fd_backward(const FdTab<C, N>& t, const T* z, T*
 #pragma unroll
   for (int j = 0; j < H; ++j) {
     const T u = chain<C, T, SHORT, HE>(t.Fb + j * HE, z);
-    const T v = chain<C, T, SHORT, H>(t.Gb + j * H, z + HE);
-    out[j] = finish(add_lazy(u, v));
-    out[N - 1 - j] = finish(sub_lazy(u, v));
+    T lo, hi;
+    chain_sum<SHORT, N, false>(t.Gb + j * H, z + HE, u, lo, hi);
+    out[j] = finish(lo);
+    out[N - 1 - j] = finish(hi);
   }
   if (N % 2) out[H] = finish(chain<C, T, SHORT, HE>(t.Fb + H * HE, z));
 }
@@ -816,15 +841,15 @@ __device__ __forceinline__ void general_body(const ApplyJob<S, T>& a, const Tab<
   __syncthreads();
   // t = Dc^T_x v1 (+ m u) + Dc^T_y v2 + Dc^T_z v3 at points (pa, pb, q), then S^T along z
   {
-    T tq[N];
-    Fold<T, N, true, SH>(d3).apply(tab.eDt, tq); // Dc^T_z v3 along this pencil
+    T s[N], tq[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       const int l = pa + N * pb + N2 * q;
-      T s = buf1[l * CB + c];
-      if (HELM) s = add_lazy(s, U[q]);
-      tq[q] = finish(add_lazy(add_lazy(s, buf2[l * CB + c]), tq[q]));
+      s[q] = buf1[l * CB + c];
+      if (HELM) s[q] = add_lazy(s[q], U[q]);
+      s[q] = add_lazy(s[q], buf2[l * CB + c]);
     }
+    Fold<T, N, true, SH>(d3).add_to(s, tab.eDt, tq); // Dc^T_z v3 along this pencil
     T out[N];
     Fold<T, N, false, SH>(tq).apply(tab.eSt, out);
 #pragma unroll

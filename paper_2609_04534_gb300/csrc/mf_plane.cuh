@@ -408,12 +408,13 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
   __syncthreads();
 #pragma unroll (N == 2 ? 2 : 1)
   for (int i = 0; i < N; ++i) { // pencils (i, j = p)
-    T v3[N], tq[N], out[N];
+    T v3[N], s[N], tq[N], out[N];
 #pragma unroll
-    for (int q = 0; q < N; ++q) v3[q] = B[(i + N * p + N2 * q) * CB];
-    Fold<T, N, true, SH>(v3).apply(tab.eDt, tq);
-#pragma unroll
-    for (int q = 0; q < N; ++q) tq[q] = finish(add_lazy(A[(i + N * p + N2 * q) * CB], tq[q]));
+    for (int q = 0; q < N; ++q) {
+      v3[q] = B[(i + N * p + N2 * q) * CB];
+      s[q] = A[(i + N * p + N2 * q) * CB];
+    }
+    Fold<T, N, true, SH>(v3).add_to(s, tab.eDt, tq);
     Fold<T, N, false, SH>(tq).apply(tab.eSt, out);
 #pragma unroll
     for (int k = 0; k < N; ++k) A[(i + N * p + N2 * k) * CB] = out[k];

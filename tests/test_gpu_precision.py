@@ -1,7 +1,8 @@
-"""Accuracy of the double-float kernels against the oracle's 64-bit arithmetic, by the relative L2
-error over several inputs: not larger than with the full-length products (fma in mf_dd.cuh), whose
-errors on these inputs are listed.  The computation is deterministic; the margin covers the
-order of the CG scalars' 64-bit sums (1e-16 of errors of 1e-14)."""
+"""Accuracy of the apply kernels against the oracle's 64-bit arithmetic, by the relative L2
+error over several inputs: not larger than with the full-length products (fma in mf_dd.cuh) and,
+in FP32, with products contracted into sums, whose errors on these inputs are listed.  The
+computation is deterministic; the margin covers the order of the CG scalars' 64-bit sums (1e-16 of
+errors of 1e-14)."""
 import numpy as np
 import pytest
 import torch
@@ -64,3 +65,11 @@ def test_cg_vectors_in_double_float_lose_nothing(oracle, geom, k):
 @pytest.mark.parametrize("geom,k", list(APPLY))
 def test_apply_with_truncated_input_loses_nothing(oracle, geom, k):
     assert apply_error(oracle, geom, k, mf.MF_FP64) <= 1.001 * APPLY[geom, k]
+
+
+FP32 = {("cart", 2): 1.2651e-07, ("shear", 2): 1.3249e-07}  # one rounding per product and sum
+
+
+@pytest.mark.parametrize("geom,k", list(FP32))
+def test_fp32_products_go_into_sums_by_one_rounding(oracle, geom, k):
+    assert apply_error(oracle, geom, k, mf.MF_FP32) <= 1.001 * FP32[geom, k]
