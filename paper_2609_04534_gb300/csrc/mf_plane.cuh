@@ -274,6 +274,31 @@ __device__ __forceinline__ void plane_y(const EoTab<C, N>& m, T (&u)[N][N]) {
   }
 }
 
+// A thread's part of <p, A p> over its plane: every row of n points is summed like a pencil of
+// general_body, and the rows are joined in double-float (FP32) or double.  (A plain FP32 sum over n^2
+// points lost 1e-6 of a sum of one large and many small terms.)
+template <typename T>
+struct RowSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(T row) { s += to_double(finish(row)); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct RowSum<float> {
+  AccF acc;
+  __device__ __forceinline__ void add(float row) { acc.add2(row, 0.0f); }
+  __device__ __forceinline__ double value() const { return acc.value(); }
+};
+template <>
+struct RowSum<f2> {
+  AccF acc;
+  __device__ __forceinline__ void add(f2 row) {
+    acc.add2(row.x, 0.0f);
+    acc.add2(row.y, 0.0f);
+  }
+  __device__ __forceinline__ double value() const { return acc.value(); }
+};
+
 // General cells (see general_body).  Stages: plane k = p: load, S along x and y | plane j = p:
 // S along z and the z-derivative | plane q = p: x- and y-derivatives, metric, Dc^T along x and
 // y | plane j = p: Dc^T along z, S^T along z | plane k = p: S^T along y and x, store.
@@ -318,7 +343,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
   }
   __syncthreads();
   const bool fuse = a.cg.st != nullptr;
-  T pap = T(0);
+  RowSum<T> pap;
   { // plane q = p: u holds U, then Dc^T_x v1 (+ m U), row by row; d2 the y-derivatives, then v2
     T u[N][N], d2[N][N];
 #pragma unroll
@@ -349,7 +374,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
       gp = a.geom + ((cell.t * NC) * (long long)N3 + (long long)N2 * p) * BL + cell.lane;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      T d1[N], mu[N];
+      T d1[N], mu[N], row = T(0);
       Fold<T, N, true, SH>(u[j]).apply(tab.eD, d1);
       float syz = 0.f, pyz = 0.f, spz = 0.f;
       if constexpr (CURVED && IsF32<T>::value) {
@@ -388,12 +413,13 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
         d1[i] = v1;
         d2[j][i] = v2;
         B[l * CB] = v3;
-        if (fuse) pap = fma(e1, v1, fma(e2, v2, fma(e3, v3, pap)));
+        if (fuse) row = fma(e1, v1, fma(e2, v2, fma(e3, v3, row)));
         if (HELM) {
           mu[i] = m * u[j][i];
-          if (fuse) pap = fma(u[j][i], mu[i], pap);
+          if (fuse) row = fma(u[j][i], mu[i], row);
         }
       }
+      if (fuse) pap.add(row);
       T out[N];
       Fold<T, N, true, SH>(d1).apply(tab.eDt, out);
 #pragma unroll
@@ -432,7 +458,7 @@ __device__ __forceinline__ void general_plane(const ApplyJob<S, T>& a, const Tab
   }
   if (fuse) {
     __shared__ double red[NT];
-    red[threadIdx.x] = to_double(finish(pap));
+    red[threadIdx.x] = pap.value();
     __syncthreads();
     cta_partial_after_barrier<NT>(red, a.cg.partials, cta);
   }
