@@ -1,10 +1,13 @@
-"""CG on meshes large enough for the plane kernels (mf_plane.cuh)."""
+"""CG on meshes large enough for the plane kernels (mf_plane.cuh): FP32 from 304 tiles, double-float
+from 2048, with tile counts that leave the last FP32 CTA one tile past the end."""
 import numpy as np
 import pytest
 import torch
 
 import paper_2609_04534_gb300 as mf
-from tests._gpu import SHEAR_A, DevOp
+from paper_2609_04534_gb300 import inputs
+from tests._gpu import SHEAR_A, DevOp, rel_max
+from tests.test_gpu_cg import consistent, solve
 
 pytestmark = pytest.mark.gpu
 
@@ -53,3 +56,35 @@ def test_pairing_of_one_large_and_many_small_terms():
     plane, pencil = one_step(d, b, 0), one_step(d, b, 1)
     d.close()
     assert abs(plane / pencil - 1.0) <= (n - 1) * 2.0**-24, plane / pencil - 1.0
+
+
+FP32, FP64 = mf.MF_FP32, mf.MF_FP64
+CASES = ([(FP32, k, (28, 27, 13), g) for k in range(1, 6) for g in ("curved", "shear")] +
+         [(FP32, k, (28, 27, 13), "cart") for k in (2, 6)] +
+         [(FP64, 1, (44, 43, 33), g) for g in ("cart", "curved", "shear")] +
+         [(FP64, 2, (44, 43, 33), g) for g in ("cart", "shear")])
+
+
+@pytest.mark.parametrize("prec,k,dims,geom", CASES)
+def test_split_forms_match_the_pencil_kernels_and_the_assembled_form(prec, k, dims, geom):
+    """Six iterations: the split-dual forms (with the direction formed by its own kernel, and by the
+    apply at load) on plane kernels, the same on pencil kernels, and the assembled form give the same
+    residuals and iterate up to the rounding of the scalars, whose effect grows by less than an order
+    per iteration; iterates stay consistent."""
+    for kind, bc in ((mf.MF_LAPLACE, 1), (mf.MF_HELMHOLTZ, 0)):
+        d = DevOp(*dims, k, geom, kind, 1.0, prec, bc)
+        b = d.native_from_unique(inputs.random_unique(*dims, k, 23))
+        its, tol = 6, 1e-4 if prec == FP32 else 1e-11
+        mf.mf_operator_set_variant(d.op, 0)
+        runs = [solve(d, b, 0.0, its, 0, hist_cap=its + 2, cg_form=f)
+                for f in (mf.MF_CG_SPLIT_DUAL, mf.MF_CG_SPLIT_DUAL_FUSED, mf.MF_CG_ASSEMBLED)]
+        mf.mf_operator_set_variant(d.op, 1)
+        runs += [solve(d, b, 0.0, its, 0, hist_cap=its + 2, cg_form=f)
+                 for f in (mf.MF_CG_SPLIT_DUAL, mf.MF_CG_SPLIT_DUAL_FUSED)]
+        x0, st0, h0 = runs[0]
+        assert st0["iterations"] == its and consistent(d, x0)
+        for x, st, h in runs[1:]:
+            assert st["iterations"] == its and consistent(d, x)
+            np.testing.assert_allclose(h[:its + 1], h0[:its + 1], rtol=tol, atol=0)
+            assert rel_max(d.unique_from_native(x), d.unique_from_native(x0)) <= tol
+        d.close()
