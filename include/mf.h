@@ -380,10 +380,13 @@ mf_status mf_cg_record_history(double* hist_host, int cap);
  * free (a request that does not fit yet does not block smaller ones behind it).  An admitted
  * request keeps its geometry, vectors and CG state resident in its arena block.  Its set-up,
  * the outer steps of defect correction and its finish run on its slot's CUDA stream; its CG
- * iterations run in a continuous batch: every active request of the same degree, path,
- * operator kind, vector precision and launch configuration takes part in one batched launch per
- * kernel of the (split-dual) CG iteration -- apply, update, direction -- in chunks of
- * chunk_iterations, and requests join and leave the batch between chunks.  The batched apply
+ * iterations run in a continuous batch: the requests of one class -- the same degree, path,
+ * operator kind, vector precision and launch configuration -- that are ready at the same time
+ * share one batched launch per kernel of the (split-dual) CG iteration -- apply, update,
+ * direction -- in chunks of chunk_iterations, and requests join and leave the batch between
+ * chunks.  A request that is ready alone in its class runs the same chunk as a graph of its
+ * own.  The launch configuration depends on the mesh size as well: double-float requests of up to 64
+ * tiles of 32 cells and larger ones are different classes.  The batched apply
  * is one persistent launch: the CTAs that fit the GPU at once loop over the CTA-sized work
  * units of all members.  Requests whose own apply takes more than 1024 CTAs run their own
  * graph chunks (they fill the GPU alone).  Each request's
@@ -447,6 +450,8 @@ mf_status mf_batch_cancel(mf_server* server, uint64_t ticket);
 /* Waits (bounded) until no request is queued or running; MF_ERR_TIMEOUT otherwise. */
 mf_status mf_server_drain(mf_server* server, double timeout_s);
 mf_status mf_server_stats(mf_server* server, mf_server_stats_t* out);
+/* Chunks that ran as batched launches since the server was created, and their members in all. */
+mf_status mf_server_batch_counts(mf_server* server, int64_t* chunks, int64_t* members);
 /* Cancels outstanding work, waits for the slot streams and frees host resources. */
 void mf_server_destroy(mf_server* server);
 

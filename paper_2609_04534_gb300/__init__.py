@@ -150,6 +150,7 @@ def lib() -> C.CDLL:
     L.mf_batch_cancel.argtypes = [vp, C.c_uint64]
     L.mf_server_drain.argtypes = [vp, d]
     L.mf_server_stats.argtypes = [vp, C.POINTER(mf_server_stats_t)]
+    L.mf_server_batch_counts.argtypes = [vp, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
     L.mf_server_destroy.argtypes = [vp]
     L.mf_server_destroy.restype = None
     _lib = L
@@ -413,6 +414,13 @@ def mf_server_stats(server) -> dict:
     st = mf_server_stats_t()
     _check(lib().mf_server_stats(server, C.byref(st)))
     return {f: getattr(st, f) for f, _ in mf_server_stats_t._fields_}
+
+
+def mf_server_batch_counts(server) -> tuple:
+    """(chunks that ran as batched launches, their members in all)"""
+    chunks, members = C.c_int64(), C.c_int64()
+    _check(lib().mf_server_batch_counts(server, C.byref(chunks), C.byref(members)))
+    return chunks.value, members.value
 
 
 def mf_server_destroy(server) -> None:
