@@ -45,8 +45,11 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), unsigned blocks, int th
   cfg.stream = s;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cfg.attrs = &attr;
-  cfg.numAttrs = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, Params(std::forward<Args>(args))...);
+  const cudaError_t asked = cudaStreamIsCapturing(s, &cap);
+  cfg.numAttrs = asked == cudaSuccess && cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, Params(std::forward<Args>(args))...);
+  if (e != cudaSuccess || asked != cudaSuccess) (void)cudaGetLastError(); // reported here, not by the next check as well
+  return e;
 }
 
 } // namespace mf
