@@ -881,7 +881,7 @@ static mf_status eng_chunk(SolverEngine* e) {
   cudaStream_t s = e->s;
   mf_status st;
   const int left = e->hm->st.maxit - e->hm->st.it;
-  if (e->direct > 0 && !e->exec && (e->direct > 1 || left <= 3 * e->chunk)) {
+  if (e->direct > 0 && !e->exec && (e->direct > 1 || left <= 3LL * e->chunk)) {
     if (e->direct > 1) --e->direct;
     const int n = e->chunk < left ? e->chunk : (left > 1 ? left : 1);
     for (int c = 0; c < n; ++c)
