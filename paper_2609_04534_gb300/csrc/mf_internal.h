@@ -145,6 +145,10 @@ struct ApplyBatch {
   int njobs;
 };
 
+// Meshes of at most this many tiles join continuous batches (a nominal 1024 CTAs of a quarter tile,
+// about two waves of two CTAs per SM): alone, those are launch- and latency-bound.
+constexpr long long BATCH_MAX_TILES = 256;
+
 // One request of a batched CG iteration (the serving loop): its operator and CG storage.
 struct BatchMember {
   const mf_operator* op;

@@ -1739,14 +1739,23 @@ constexpr int CFG_PLANE = 6;
 // FP32: from one CTA per SM (two tiles each), always where the stretch is short (n = 2;
 // Cartesian up to n = 4).  Double-float: from 2048 tiles (Q2 Cartesian 16^3 6.4 against 4.4 us, 32^3
 // 12.0 against 12.9).
+template <typename T, int N, int PATH>
+constexpr long long plane_from_tiles() {
+  return std::is_same<T, dd>::value ? 2048 : (N == 2 || (PATH == PATH_CARTESIAN && N <= 4) ? 0 : 304);
+}
 template <typename T, int N>
 static bool use_plane(const mf_operator* op) {
-  const bool built = op->path == PATH_CARTESIAN ? UsePlane<T, N, PATH_CARTESIAN>::value
-                                                : (op->path == PATH_AFFINE ? UsePlane<T, N, PATH_AFFINE>::value
-                                                                           : UsePlane<T, N, PATH_CURVED>::value);
-  if (!built) return false;
-  if (std::is_same<T, dd>::value) return op->g.ntiles >= 2048;
-  return N == 2 || (op->path == PATH_CARTESIAN && N <= 4) || op->g.ntiles >= 304;
+  const long long t = op->g.ntiles;
+  if (op->path == PATH_CARTESIAN)
+    return UsePlane<T, N, PATH_CARTESIAN>::value && t >= plane_from_tiles<T, N, PATH_CARTESIAN>();
+  if (op->path == PATH_AFFINE) return UsePlane<T, N, PATH_AFFINE>::value && t >= plane_from_tiles<T, N, PATH_AFFINE>();
+  return UsePlane<T, N, PATH_CURVED>::value && t >= plane_from_tiles<T, N, PATH_CURVED>();
+}
+// Whether a batch's members (at most BATCH_MAX_TILES) ever take a plane kernel: FP32 where planes have no
+// line.  The others are not built.
+template <typename T, int N, int PATH>
+constexpr bool plane_in_batch() {
+  return UsePlane<T, N, PATH>::value && plane_from_tiles<T, N, PATH>() <= BATCH_MAX_TILES;
 }
 // Small meshes take variant 1's smaller CTAs: FP32 below the plane kernels' line, double-float
 // up to 64 tiles (curved Q4 8^3 12.4 -> 8.4 us, Q6 19.7 -> 13.1, Cartesian Q6 11.3 -> 8.3; at 128
@@ -1960,16 +1969,17 @@ static mf_status batch_launch_v(const mf_operator* op0, const void* jobs_dev, co
     using P = PlaneCfg<T, N>;
     h.threads = P::NT;
     h.smem = (op0->path == PATH_CARTESIAN ? 1 : 2) * sizeof(T) * N * N * N * P::CB;
-    if constexpr (UsePlane<T, N, PATH_CARTESIAN>::value)
+    if constexpr (plane_in_batch<T, N, PATH_CARTESIAN>())
       if (op0->path == PATH_CARTESIAN)
         h.kernel = helm ? apply_cartesian_plane_batch<S, T, N, true> : apply_cartesian_plane_batch<S, T, N, false>;
-    if constexpr (UsePlane<T, N, PATH_AFFINE>::value)
+    if constexpr (plane_in_batch<T, N, PATH_AFFINE>())
       if (op0->path == PATH_AFFINE)
         h.kernel =
             helm ? apply_general_plane_batch<S, T, N, false, true> : apply_general_plane_batch<S, T, N, false, false>;
-    if constexpr (UsePlane<T, N, PATH_CURVED>::value)
+    if constexpr (plane_in_batch<T, N, PATH_CURVED>())
       if (op0->path == PATH_CURVED)
         h.kernel = helm ? apply_general_plane_batch<S, T, N, true, true> : apply_general_plane_batch<S, T, N, true, false>;
+    if (!h.kernel) return set_error(MF_ERR_UNSUPPORTED, "batch: members above %lld tiles", BATCH_MAX_TILES);
   } else {
     h.threads = C::NT;
     h.smem = (op0->path == PATH_CARTESIAN ? (MF_CART_FD ? 1 : 2) : 3) * sizeof(T) * N * N * N * C::CB;

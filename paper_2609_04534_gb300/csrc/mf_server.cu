@@ -100,10 +100,6 @@ __global__ void random_unique_kernel(double* u, long long n, unsigned long long 
 
 enum Stage { ST_QUEUED = 0, ST_SOLVING = 1, ST_FINISHING = 2, ST_DONE = 3 };
 
-// Requests whose apply launches at most this many CTAs join continuous batches (about two
-// waves of two CTAs per SM on 152 SMs).
-constexpr long long BATCH_MAX_CTAS = 1024;
-
 struct Job {
   uint64_t ticket = 0;
   mf_request req{};
@@ -240,9 +236,7 @@ mf_status job_start(mf_server* sv, Job* j, Slot& sl, HostMirror* hm) {
   // CTAs at most: those are launch- and latency-bound alone, and batched with others they
   // share launches.  A larger request fills the GPU by itself and runs its own graph chunks
   // (batched with small ones it would hold them to its own chunk time).
-  // (a nominal count: launch configurations put 4 to 64 cells in one CTA)
-  const long long ctas = j->op->g.ntiles * 4;
-  j->eng.external = sv->cfg.batching >= 0 && ctas <= BATCH_MAX_CTAS;
+  j->eng.external = sv->cfg.batching >= 0 && j->op->g.ntiles <= BATCH_MAX_TILES;
   if ((st = engine_start(&j->eng))) return st;
   // every advance finishes or moves the iteration count forward by a chunk
   j->max_steps = 2LL * ((long long)j->req.maxit / j->eng.chunk + 2) * (j->eng.max_outer + 2) + 16;

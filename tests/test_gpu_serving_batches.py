@@ -42,3 +42,27 @@ def test_staggered_requests_of_one_class_run_in_batches():
     finally:
         mf.mf_server_destroy(sv)
     assert r1["iterations"] == res[3]["iterations"] and np.array_equal(x1, outs[3])
+
+
+@pytest.mark.parametrize("geometry,k", [(mf.MF_AFFINE, 1), (mf.MF_AFFINE, 2), (mf.MF_AFFINE, 3), (mf.MF_CURVED_SIN, 1)])
+def test_batched_plane_kernels_match_solo_solves(geometry, k):
+    """Mixed requests whose FP32 inner CG runs on plane kernels at any size (Cartesian of degrees 1
+    to 3, general of degree 1), ragged meshes with odd tile counts, in one batch: bitwise the solutions
+    of the requests alone."""
+    reqs = [dict(nx=5 + 2 * i, ny=7, nz=3 + i, degree=k, geometry=geometry, rhs=mf.MF_RHS_RANDOM, seed=40 + i, mixed=1)
+            for i in range(6)]
+    sv, arena = make_server(slots=16)
+    try:
+        res, xs = run(sv, [mf.make_request(**p) for p in reqs])
+        chunks, members = mf.mf_server_batch_counts(sv)
+    finally:
+        mf.mf_server_destroy(sv)
+    assert members >= 2 * chunks > 0
+    for p, r, x in zip(reqs, res, xs):
+        sv, arena = make_server(slots=1, batching=-1)
+        try:
+            (r1,), (x1,) = run(sv, [mf.make_request(**p)])
+        finally:
+            mf.mf_server_destroy(sv)
+        assert r["status"] == r1["status"] == mf.MF_OK and r1["iterations"] == r["iterations"]
+        assert np.array_equal(x1, x), p
