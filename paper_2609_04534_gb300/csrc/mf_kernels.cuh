@@ -1737,8 +1737,11 @@ constexpr int CFG_PLANE = 6;
 // Planes need enough CTAs: one CTA's pass is a long serial stretch per thread (FP32 curved Q4:
 // 9.1 us on any mesh up to 12^3 cells, the pencil kernel 3.7; at 24^3, 216 CTAs, 13.3 against 16.4).
 // FP32: from one CTA per SM (two tiles each), always where the stretch is short (n = 2;
-// Cartesian up to n = 4).  Double-float: from 2048 tiles (Q2 Cartesian 16^3 6.4 against 4.4 us, 32^3
-// 12.0 against 12.9).
+// Cartesian up to n = 4).  Double-float: from 2048 tiles (split apply, us, plane / pencil: Q2
+// Cartesian 32^3, 1024 tiles, 14.6 / 10.0; 40^3, 2000 tiles, 17.1 / 17.7; 48^3 26.3 / 27.9; 64^3 56.6 / 64.5;
+// Q2 sheared 22.0 / 21.0, 35.6 / 38.9, 56.8 / 62.7, 133 / 145; Q1 curved 9.5 / 7.3, 11.2 / 11.0, 15.7 / 17.2,
+// 36.8 / 40.5).  On CG's double-float vectors planes win from about 500 tiles (Q2 Cartesian 32^3 12.6 /
+// 15.7), but one line serves both.
 template <typename T, int N, int PATH>
 constexpr long long plane_from_tiles() {
   return std::is_same<T, dd>::value ? 2048 : (N == 2 || (PATH == PATH_CARTESIAN && N <= 4) ? 0 : 304);
@@ -1760,20 +1763,23 @@ constexpr bool plane_in_batch() {
 // Small meshes take variant 1's smaller CTAs: FP32 below the plane kernels' line, double-float
 // up to 64 tiles (curved Q4 8^3 12.4 -> 8.4 us, Q6 19.7 -> 13.1, Cartesian Q6 11.3 -> 8.3; at 128
 // tiles curved Q4 19.9 against 21.6).  Above, double-float (split apply, ms at ~17M DoFs, base
-// configuration -> the chosen one).  Cartesian: Q3 0.256 -> 0.181, Q4 0.311 -> 0.228, Q5 0.291 ->
-// 0.224, Q6 0.387 -> 0.315, Q7 0.379 -> 0.350, Q8 0.507 -> 0.428.  Affine: Q3 0.392 -> 0.348, Q4
-// 0.560 -> 0.468, Q6 0.766 -> 0.687, the others stay.  Curved: Q2 0.515 -> 0.411, Q3 0.438 -> 0.419,
-// Q4 (Laplace) 0.513 -> 0.483, Q5 0.646 -> 0.623, Q6 (Laplace) 0.771 -> 0.734, the others stay.
+// configuration -> the chosen one).  Cartesian: Q3 0.174 -> 0.147, Q4 0.221 -> 0.178, Q5 0.218 ->
+// 0.196, Q6 0.305 -> 0.255, Q7 0.219 -> 0.210, Q8 0.392 -> 0.347.  Affine: Q3 0.362 -> 0.335, Q4
+// 0.459 -> 0.397, Q6 0.683 -> 0.632, the others stay.  Curved: Q2 0.361 -> 0.354 (Helmholtz 0.428 ->
+// 0.364), Q3 0.367 -> 0.342, Q4 (Laplace) 0.453 -> 0.408, Q5 (Helmholtz) 0.601 -> 0.577, Q6 (Laplace)
+// 0.691 -> 0.681, the others stay (Q8 would gain above 20^3 cells and lose below).  CG's apply on double-float
+// vectors takes the same: there the choice loses in Cartesian Q7 (0.216 -> 0.229) and gains or is even
+// elsewhere (curved Q4 0.488 -> 0.469; with variant 4, whose 40 registers spill there, 0.528).
 template <typename T, int N>
 static int pencil_config(const mf_operator* op) {
   if (IsF32<T>::value) return N <= (op->path == PATH_CARTESIAN ? 7 : 6) && op->g.ntiles < 304 ? 1 : 0;
   if (!std::is_same<T, dd>::value) return 0;
   if (op->g.ntiles <= 64) return 1;
-  if (op->path == PATH_CARTESIAN) return N == 7 || N == 9 ? MF_VARIANT_OCCUPANCY : (N >= 4 ? MF_VARIANT_SMALL_CTA : 0);
+  if (op->path == PATH_CARTESIAN) return N >= 7 ? MF_VARIANT_OCCUPANCY : (N >= 4 ? MF_VARIANT_SMALL_CTA : 0);
   if (op->path == PATH_AFFINE) return N == 4 ? MF_VARIANT_SMALL_CTA : (N == 5 || N == 7 ? MF_VARIANT_OCCUPANCY : 0);
-  if (N == 3 || (N == 5 && op->kind == MF_LAPLACE)) return MF_VARIANT_SMALL_CTA;
-  if (N == 4 || N == 6) return 1;
-  return N == 7 && op->kind == MF_LAPLACE ? MF_VARIANT_OCCUPANCY : 0;
+  if (N == 3) return MF_VARIANT_SMALL_CTA;
+  if (N == 4 || (N == 6 && op->kind == MF_HELMHOLTZ)) return 1;
+  return (N == 5 || N == 7) && op->kind == MF_LAPLACE ? MF_VARIANT_OCCUPANCY : 0;
 }
 // The configuration of a pencil / plane launch with this variant (the tensor-core variant's
 // operators run variant 0 where their vectors are not plain doubles).
