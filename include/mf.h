@@ -108,9 +108,10 @@ mf_status mf_operator_info(const mf_operator* op, mf_info* info);
 mf_status mf_operator_setup(mf_operator* op, void* workspace_dev, size_t bytes, void* stream);
 
 /* Autotuner: times each launch configuration of the apply kernel (variant 0: the configuration
- * measured fastest for the operator's degree, path and precision -- one thread per plane of a
- * cell for MF_FP32 up to degree 5 (6 on Cartesian meshes) and MF_FP64 of degree 1 and 2, else one
- * of the pencil configurations; variant 1: one thread per pencil, half of the base configuration's
+ * measured fastest for the operator's degree, path, precision and mesh size: one thread per plane
+ * of a cell for the FP32 view up to degree 5 (6 on Cartesian meshes) from 304 tiles of 32 cells (of any
+ * size at degree 1 and on Cartesian meshes up to degree 3), and for the double-float view at degree 1
+ * and, except on curved meshes, 2 from 2048 tiles; else one of the pencil configurations; variant 1: one thread per pencil, half of the base configuration's
  * n^2 x CB threads per CTA, registers capped for three CTAs per SM; variant 2: half the cells per
  * CTA, no register cap; variant 3, for
  * MF_FP64 operators on an axis-aligned affine mesh of degree 1..3 only: the tensor-core

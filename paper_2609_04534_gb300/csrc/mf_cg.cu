@@ -425,7 +425,8 @@ __global__ void __launch_bounds__(RED_THREADS, update_minb(sizeof(T) == 4, N))
 }
 // CTAs of an update: one warp per x-pencil unit up to one wave of resident CTAs, whose warps then
 // loop.  Several waves each paid the launch and the reduction's tail: with the folded alpha, a CG
-// iteration of Q4 FP32 on 24^3 (vectors in L2) went from 46.7 to 36.7 us, FP64 103.9 to 89.6.
+// iteration of Q4 FP32 on 24^3 (vectors in L2) went from 46.7 to 36.7 us, FP64 103.9 to 89.6.  The wave
+// is that of GB300's 152 SMs by constant, so that the order of the sums does not depend on the device.
 static int update_ctas(const mf_operator* op, int elem) {
   const long long units = op->g.ntiles * op->n * op->n, need = (units + RED_THREADS / 32 - 1) / (RED_THREADS / 32);
   const int wave = 152 * update_minb(elem == 4, op->n);

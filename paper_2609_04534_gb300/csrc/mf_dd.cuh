@@ -5,9 +5,9 @@
 // Building blocks are the classical error-free transformations: Knuth's TwoSum
 // (s + e = a + b exactly) and the FMA-based TwoProd (p + e = a * b exactly, e = fma(a, b, -p)).
 // fma() below accumulates a*b + c without renormalising; finish() renormalises a chain result
-// with Dekker's FastTwoSum.  Conversions to and from double split the IEEE bit pattern with
-// integer operations (on the way in) or by the otherwise idle FP64 pipe (on the way out), so the
-// hot loop issues no FP64 instruction.
+// with Dekker's FastTwoSum.  A double is split by integer operations on its bits; a result is joined
+// by the otherwise idle FP64 pipe (two conversions and an add per stored value).  The arithmetic
+// between them issues no FP64 instruction.
 #pragma once
 #include <cstring>
 
@@ -63,7 +63,8 @@ __device__ __forceinline__ dd fma(dd a, dd b, dd c) {
 // difference p - v and TwoProd's error a.hi b.hi - p are taken together, as a.hi b.hi - v in one
 // fma, and the cross terms go straight into lo.  lo is rounded once more per term, so it is used
 // only where the rounded conversion of double input outweighs that (ShortProducts, mf_kernels.cuh; split
-// apply, FP64: Q4 curved 52^3 0.537 -> 0.509 ms, Q4 Cartesian 52^3 0.226 -> 0.212).
+// apply of doubles, against fma() everywhere: Q4 curved 52^3 0.438 -> 0.409 ms, Q4 Cartesian 52^3 0.189 ->
+// 0.177, Q7 Cartesian 33^3 0.294 -> 0.282).
 __device__ __forceinline__ dd fma_short(dd a, dd b, dd c) {
   const float p = a.hi * b.hi;
   const float s = __fadd_rn(c.hi, p);

@@ -92,8 +92,8 @@ struct CgState {
 // CG step carried by an apply launch (the split-dual iteration of Sec. 4): with st set, the
 // apply writes the split product y = A_K p per cell (no duplicate summation) and each CTA
 // writes its part of <p, y> over all copies -- the pairing of a consistent with a split
-// vector, Lemma 1 -- to partials[blockIdx.x]; a one-CTA kernel then folds the partials and
-// forms alpha = <r, r> / <p, y>.  The input is p = x; with update_p the apply instead reads r
+// vector, Lemma 1 -- to partials[blockIdx.x]; the update (or, above 16384 of them, a one-CTA
+// kernel) then folds the partials and forms alpha = <r, r> / <p, y>.  The input is p = x; with update_p the apply instead reads r
 // and the previous direction p and forms p = r + beta p at load (written back in place).
 template <typename S>
 struct CgFuse {

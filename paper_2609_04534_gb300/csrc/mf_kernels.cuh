@@ -209,9 +209,10 @@ struct Fold {
 };
 
 // Whether a kernel carries dd_from_double's general form in line (its registers) or calls it
-// (its code).  Split apply, FP64, ms in line / called: Cartesian Q3 64^3 0.153 / 0.162, Q4 52^3 0.193 /
-// 0.198, Q7 33^3 0.297 / 0.286, Q8 30^3 0.374 / 0.345; curved Q1 120^3 0.251 / 0.221, Q3 64^3 0.387 /
-// 0.370.
+// (its code).  Split apply, FP64, ms in line / called: Cartesian Q3 64^3 0.146 / 0.152, Q4 52^3 0.177 /
+// 0.184, Q5 44^3 0.196 / 0.201, Q7 33^3 0.300 / 0.282, Q8 30^3 0.375 / 0.347; curved Q3 64^3 0.365 /
+// 0.341, Q4 52^3 0.411 / 0.409.  (The Q2 Cartesian plane kernel, in line with the rest, takes 0.136 against
+// 0.124 at 88^3; doubles there run on the tensor cores by default.)
 template <int N>
 struct InlineFrom { static constexpr bool cartesian = N <= 7; };
 template <bool INL, bool NEAR, typename T, typename S>

@@ -10,15 +10,16 @@
 // both give bitwise equal results.
 //
 // What bounds it: instruction fetch.  The plane's sweeps are straight-line code (their arrays are
-// registers), a few warps per scheduler run it, and at n = 5 (FP32, curved) 1.8 warps stalled on
-// fetch per issued instruction.  The pencil loops between shared memory and shared memory
-// are therefore not unrolled (Q4 curved FP32 52^3 0.099 -> 0.092 ms, Q5 44^3 0.161 -> 0.106), and
-// double-float, whose code is six times longer, uses planes only where n is 2 or 3.
-// Measured against the pencil kernels on one GB300 (split apply, ms): FP32 Q2 Cartesian 88^3
-// 0.064 -> 0.030, Q4 Cartesian 52^3 0.062 -> 0.034 (60% of HBM), Q6 Cartesian 38^3 0.074 -> 0.060,
-// Q4 curved 52^3 0.126 -> 0.092 (188 -> 114 instructions per DoF), Q4 sheared 52^3 0.125 -> 0.076;
-// FP64 (double-float) Q1 Cartesian 120^3 0.148 -> 0.115, Q2 Cartesian 88^3 0.220 -> 0.166, Q1
-// curved 120^3 0.277 -> 0.237, Q2 sheared 88^3 0.531 -> 0.368.
+// registers), a few warps per scheduler run it, and at n = 5 (FP32, curved, 48^3) 0.95 warps are stalled
+// on fetch per issued instruction, more than for any other reason; 56% of issue slots are used.
+// The pencil loops between shared memory and shared memory are therefore not unrolled (with them
+// unrolled Q4 curved FP32 52^3 took 0.099 ms, Q5 44^3 0.161), and double-float, whose code is six times
+// longer, uses planes only where n is 2 or 3.
+// Measured against the pencil kernels on one GB300 (split apply, ms, pencil -> plane): FP32 Q2 Cartesian
+// 88^3 0.041 -> 0.025, Q4 Cartesian 52^3 0.038 -> 0.030 (69% of HBM), Q6 Cartesian 38^3 0.054 -> 0.053,
+// Q4 curved 52^3 0.117 -> 0.089 (114 instructions per DoF), Q5 curved 44^3 0.116 -> 0.103, Q4 sheared
+// 52^3 0.093 -> 0.072; FP64 (double-float) Q1 Cartesian 120^3 0.114 -> 0.092, Q2 Cartesian 88^3 0.161 ->
+// 0.136, Q1 curved 120^3 0.242 -> 0.220, Q2 sheared 88^3 0.370 -> 0.332.
 #pragma once
 
 namespace mf {
